@@ -156,10 +156,13 @@ typedef struct {
     int32_t storage;   /* lbm_storage */
     int32_t wall_values; /* lbm_wall_values */
     int32_t time_block;  /* time steps fused into one kernel launch:
-                            0  library default: LBM_TIME_BLOCK where it is the
-                               faster form (supported, lambda = mu, at least 2^21
-                               nodes, at most one boundary node per 800 nodes that
-                               is not on a box edge or crack face); else 1
+                            0  library default, the faster form: with FP32 storage
+                               and two buffers several steps per launch, by the
+                               strip kernel of LBM_TIME_BLOCK (lambda = mu, at least
+                               2^21 nodes, nx >= 128, at most one boundary node per
+                               800 nodes that is not on a box edge or crack face)
+                               or in register tiles (the other lattices, unless
+                               walls are everywhere); else 1
                             1  one launch per step (bulk and boundary-list kernels)
                             LBM_TIME_BLOCK  temporal blocking: each launch carries
                                LBM_TIME_BLOCK steps (4 when lambda != mu, whose
@@ -188,7 +191,7 @@ typedef struct {
     float bytes_per_update; /* algorithmic HBM bytes per interior lattice update */
     int64_t kernel_launches; /* kernels this handle has launched so far */
     int32_t time_block;      /* steps per launch in use: 1, LBM_TIME_BLOCK, or 4
-                                (temporal blocking with lambda != mu) */
+                                (several steps per launch with lambda != mu) */
     int32_t streaming;       /* lbm_streaming in use */
 } lbm_info;
 
@@ -213,7 +216,10 @@ lbm_status lbm_geom_build(const lbm_geom *geom, uint8_t *node_type, lbm_link *li
                           int64_t cap, int64_t *nlinks);
 
 /* Device bytes a handle for `desc` needs (distributions, displacement,
- * tables, field staging).  Host tables are validated as in lbm_create. */
+ * tables, field staging).  Host tables are validated as in lbm_create.  The
+ * tables of the register tiles come on top: lbm_create allocates them itself
+ * (about 100 bytes per boundary node and 32 per tile) and, if it cannot,
+ * steps one step per launch. */
 lbm_status lbm_workspace_size(const lbm_desc *desc, uint64_t *bytes);
 
 /* Create a solver: validates and classifies the tables on the host, copies

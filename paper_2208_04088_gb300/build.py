@@ -35,7 +35,7 @@ def _cuda_home() -> str:
 def sources():
     cu = sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cu"))
     cpp = sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cpp"))
-    hdr = sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h"))
+    hdr = sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh")))
     hdr += [os.path.join(INC, f) for f in os.listdir(INC) if f.endswith(".h")]
     return cu, cpp, hdr
 

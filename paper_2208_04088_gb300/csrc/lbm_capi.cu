@@ -1,5 +1,6 @@
 // lbm_capi.cu -- the C ABI of include/lbm.h: handle life cycle, device memory
 // layout, stepping (direct launches or replayed CUDA graphs), fields and probes.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -166,6 +167,18 @@ void destroy_graphs(lbm_solver *h) {
 static_assert(kGraphChunk % (2 * kWaveK) == 0 && kGraphChunk % (2 * kWaveGradK) == 0,
               "graph chunk and time block");
 
+// The fewest steps a register-tile launch is used for: two cost less there
+// than as two one-step launches (64^2 plate: 9 us against 10; lambda != mu at
+// 2048^2: 175 against 182).
+constexpr int kTileMinSteps = 2;
+
+// nsteps steps in one blocked launch: register tiles (any number up to
+// h->block) or the strip kernels (h->block).
+cudaError_t launch_blocked(lbm_solver *h, int cur, int toff, int nsteps, cudaStream_t s) {
+    return h->tile.shape >= 0 ? launch_tile(h->L, h->S, h->tile, cur, toff, nsteps, s)
+                              : launch_wave(h->L, h->S, h->wave, cur, toff, s);
+}
+
 lbm_status build_graph(lbm_solver *h, int start) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(h->cap_main, cudaStreamCaptureModeThreadLocal);
@@ -173,7 +186,7 @@ lbm_status build_graph(lbm_solver *h, int start) {
     int cur = start;
     for (int s = 0; s < kGraphChunk && e == cudaSuccess;) {
         if (h->block > 1) {
-            e = launch_wave(h->L, h->S, h->wave, cur, s, h->cap_main);
+            e = launch_blocked(h, cur, s, h->block, h->cap_main);
             s += h->block;
         } else {
             e = launch_step(h->storage, h->L, h->S, cur, s, h->cap_main, h->cap_side, h->gfork,
@@ -233,6 +246,43 @@ cudaError_t host_buffers(lbm_solver *h) {
         e = cudaMallocHost(&h->h_status, sizeof(uint32_t));
         if (e == cudaSuccess) *h->h_status = 0;
     }
+    return e;
+}
+
+// Register tiles for a handle whose state is allocated: the plan, and its
+// tables in memory of the handle's own.  Without that memory the handle keeps
+// the stepping form its workspace was laid out for.
+static cudaError_t tile_create(lbm_solver *h) {
+    if (!tile_supported()) return cudaSuccess;
+    TilePlan plan;
+    tile_choose(h->tab, h->L.grad != 0, h->L.wall_node != 0, device_sms(), &plan);
+    if (plan.shape < 0) return cudaSuccess;
+    const size_t bt = align256(plan.tiles.size() * sizeof(TileRec));
+    const size_t bp = align256(plan.pubs.size() * sizeof(uint32_t));
+    const size_t bl = align256(plan.links.size() * sizeof(TileLink));
+    TileDev &T = h->tile;
+    if (cudaMalloc(&T.mem, bt + bp + bl) != cudaSuccess) {
+        cudaGetLastError();
+        T.mem = nullptr;
+        return cudaSuccess;
+    }
+    char *m = static_cast<char *>(T.mem);
+    T.tiles = reinterpret_cast<const TileRec *>(m);
+    T.pubs = reinterpret_cast<const uint32_t *>(m + bt);
+    T.links = reinterpret_cast<const TileLink *>(m + bt + bp);
+    T.ntiles = (int)plan.tiles.size();
+    T.shape = plan.shape;
+    // pageable sources: the copies are staged before the calls return
+    cudaError_t e = cudaMemcpyAsync(m, plan.tiles.data(), plan.tiles.size() * sizeof(TileRec),
+                                    cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess && !plan.pubs.empty())
+        e = cudaMemcpyAsync(m + bt, plan.pubs.data(), plan.pubs.size() * sizeof(uint32_t),
+                            cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess && !plan.links.empty())
+        e = cudaMemcpyAsync(m + bt + bp, plan.links.data(), plan.links.size() * sizeof(TileLink),
+                            cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess) e = tile_prepare(h->L, h->S, &T);
+    h->block = h->L.grad ? kWaveGradK : kWaveK;
     return e;
 }
 
@@ -358,7 +408,14 @@ lbm_status create_prepared(const lbm_desc *desc, Tables &&tab, const Units &unit
         e = cudaMemcpyAsync(S.bcs, t.bcs.data(), t.bcs.size() * sizeof(BCDev),
                             cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = launch_reset(h->storage, h->L, S, h->stream);
-    if (e == cudaSuccess && h->block > 1) {
+    // The default takes register tiles wherever the strip kernel is not its
+    // form: 8 steps of a 64^2 plate in 17 us against 35 us one step at a time,
+    // of a 1024 x 512 plate 43 against 57, and with lambda != mu 4 steps of
+    // the 2048^2 crack in 240 us against 364 (the strip kernel: 349).
+    if (e == cudaSuccess && opt.plan_blocks <= 0 && desc->time_block == 0 && h->block == 1 &&
+        h->storage == LBM_F32 && !in_place)
+        e = tile_create(h);
+    if (e == cudaSuccess && h->block > 1 && h->tile.shape < 0) {
         if (!wave_supported(h->L)) {
             if (desc->time_block == LBM_TIME_BLOCK) {
                 set_error("lbm_create: the temporally blocked kernel is unavailable (tensor-map encoder)");
@@ -439,7 +496,8 @@ extern "C" lbm_status lbm_step(lbm_handle h, int64_t nsteps) {
                 ev.nsteps = h->block;
                 // one blocked launch as the bulk kernel; the boundary nodes are inside it
                 e = cudaEventRecord(ev.before_interior, h->stream);
-                if (e == cudaSuccess) e = launch_wave(h->L, h->S, h->wave, h->cur, (int)s, h->stream);
+                if (e == cudaSuccess)
+                    e = launch_blocked(h, h->cur, (int)s, h->block, h->stream);
                 if (e == cudaSuccess) e = cudaEventRecord(ev.after_interior, h->stream);
                 if (e == cudaSuccess) e = cudaEventRecord(ev.before_boundary, h->stream);
                 if (e == cudaSuccess) e = cudaEventRecord(ev.after_boundary, h->stream);
@@ -469,9 +527,10 @@ extern "C" lbm_status lbm_step(lbm_handle h, int64_t nsteps) {
     }
     const int64_t rest = nsteps - done;
     for (int64_t s = 0; s < rest;) {
-        if (h->block > 1 && rest - s >= h->block) {
-            e = launch_wave(h->L, h->S, h->wave, h->cur, (int)s, h->stream);
-            s += h->block;
+        const int n = (int)std::min<int64_t>(rest - s, h->block);
+        if (h->block > 1 && (n == h->block || (h->tile.shape >= 0 && n >= kTileMinSteps))) {
+            e = launch_blocked(h, h->cur, (int)s, n, h->stream);
+            s += n;
             h->launches += 1;
         } else {
             e = launch_step(h->storage, h->L, h->S, h->cur, (int)s, h->stream, nullptr, nullptr,
@@ -733,6 +792,7 @@ extern "C" lbm_status lbm_destroy(lbm_handle h) {
         cudaEventDestroy(ev.after_boundary);
     }
     if (h->owned) cudaFree(h->owned);
+    if (h->tile.mem) cudaFree(h->tile.mem);
     delete h;
     return LBM_OK;
 }

@@ -411,6 +411,14 @@ __device__ __forceinline__ int lane_cy(int k) {
 }
 
 
+// Components of c_i for the link i = opp(k), as floats (selects, no conversion).
+__device__ __forceinline__ float link_cx(int k) {
+    return (k == 1 || k == 5 || k == 8) ? -1.0f : (k == 3 || k == 6 || k == 7) ? 1.0f : 0.0f;
+}
+__device__ __forceinline__ float link_cy(int k) {
+    return (k == 2 || k == 5 || k == 6) ? -1.0f : (k == 4 || k == 7 || k == 8) ? 1.0f : 0.0f;
+}
+
 // Pieces of the cut-link rules of Sec. 4, shared by every boundary path so
 // that each evaluates the same expressions.
 //
@@ -467,29 +475,41 @@ __device__ __forceinline__ WallState wall_state(bool neu_ex, float q, float dr_x
                                                 const Lattice &L) {
     const float dvx = rmul(-L.lam_m_mu_r0, dr_x);
     const float sxx_x = radd(-pxx_x, dvx), syy_x = radd(-pyy_x, dvx), sxy_x = -pxy_x;
-    WallState s{dr_x, sxx_x, syy_x, sxy_x};
-    if (neu_ex) {
-        const float dvy = rmul(-L.lam_m_mu_r0, my_dr);
-        const float a1 = radd(1.0f, q);
-        s.drb = rfma(a1, dr_x, -rmul(q, my_dr));
-        s.sxx = rfma(a1, sxx_x, -rmul(q, radd(-my_xx, dvy)));
-        s.syy = rfma(a1, syy_x, -rmul(q, radd(-my_yy, dvy)));
-        s.sxy = rfma(a1, sxy_x, -rmul(q, -my_xy));
-    }
-    return s;
+    const float dvy = rmul(-L.lam_m_mu_r0, my_dr);
+    const float a1 = radd(1.0f, q);
+    const WallState e{rfma(a1, dr_x, -rmul(q, my_dr)), rfma(a1, sxx_x, -rmul(q, radd(-my_xx, dvy))),
+                      rfma(a1, syy_x, -rmul(q, radd(-my_yy, dvy))),
+                      rfma(a1, sxy_x, -rmul(q, -my_xy))};
+    return WallState{neu_ex ? e.drb : dr_x, neu_ex ? e.sxx : sxx_x, neu_ex ? e.syy : syy_x,
+                     neu_ex ? e.sxy : sxy_x};
 }
 
-// sigma* = t_n n n + t_t (n t + t n) + sigma_tt t t with sigma_tt of the wall state.
+// The part of sigma* = t_n n n + t_t (n t + t n) + sigma_tt t t that the boundary
+// data give (everything but sigma_tt).
+struct WallData {
+    float cxx, cyy, cxy;
+};
+
+__device__ __forceinline__ WallData wall_data(const WallFrame &w) {
+    return WallData{
+        rfma(rmul(rmul(2.0f, w.tt), w.n0), w.t0, rmul(rmul(w.tn, w.n0), w.n0)),
+        rfma(rmul(rmul(2.0f, w.tt), w.n1), w.t1, rmul(rmul(w.tn, w.n1), w.n1)),
+        rfma(w.tt, rfma(w.n0, w.t1, rmul(w.t0, w.n1)), rmul(rmul(w.tn, w.n0), w.n1))};
+}
+
+// sigma* with sigma_tt of the wall state; t0, t1: the tangent.
+__device__ __forceinline__ void wall_sigma(float t0, float t1, const WallData &d, const WallState &s,
+                                           float &sxx, float &syy, float &sxy) {
+    const float stt =
+        rfma(rmul(t1, t1), s.syy, rfma(rmul(rmul(2.0f, t0), t1), s.sxy, rmul(rmul(t0, t0), s.sxx)));
+    sxx = rfma(rmul(stt, t0), t0, d.cxx);
+    syy = rfma(rmul(stt, t1), t1, d.cyy);
+    sxy = rfma(rmul(stt, t0), t1, d.cxy);
+}
+
 __device__ __forceinline__ void wall_sigma(const WallFrame &w, const WallState &s, float &sxx,
                                            float &syy, float &sxy) {
-    const float stt = rfma(rmul(w.t1, w.t1), s.syy,
-                           rfma(rmul(rmul(2.0f, w.t0), w.t1), s.sxy, rmul(rmul(w.t0, w.t0), s.sxx)));
-    sxx = rfma(rmul(stt, w.t0), w.t0,
-               rfma(rmul(rmul(2.0f, w.tt), w.n0), w.t0, rmul(rmul(w.tn, w.n0), w.n0)));
-    syy = rfma(rmul(stt, w.t1), w.t1,
-               rfma(rmul(rmul(2.0f, w.tt), w.n1), w.t1, rmul(rmul(w.tn, w.n1), w.n1)));
-    sxy = rfma(rmul(stt, w.t0), w.t1,
-               rfma(w.tt, rfma(w.n0, w.t1, rmul(w.t0, w.n1)), rmul(rmul(w.tn, w.n0), w.n1)));
+    wall_sigma(w.t0, w.t1, wall_data(w), s, sxx, syy, sxy);
 }
 
 // Second moment of the wall equilibrium: P* = -sigma* + (lambda - mu) div u I,
@@ -507,24 +527,26 @@ __device__ __forceinline__ WallMoments wall_moments(float drb, float sxx, float 
 
 // 2 w_i f_i^eq(rho^bd, P*) of the anti-bounce-back rule for link i = opp(k).
 __device__ __forceinline__ float wall_equilibrium(int k, const WallMoments &m) {
-    const int i = k <= 4 ? (k + 1) % 4 + 1 : (k - 3) % 4 + 5;  // opp(k)
-    const float w = (i <= 4) ? (1.0f / 9.0f) : (1.0f / 36.0f);
-    const float cix = (float)(-lane_cx(k)), ciy = (float)(-lane_cy(k));
+    const float w = (k <= 4) ? (1.0f / 9.0f) : (1.0f / 36.0f);
+    const float cix = link_cx(k), ciy = link_cy(k);
     const float quad = rfma(rmul(ciy, ciy), m.ayy,
                             rfma(rmul(rmul(2.0f, cix), ciy), m.pxy, rmul(rmul(cix, cix), m.axx)));
     const float con = rmul(4.5f, rfma(-radd(m.axx, m.ayy), 1.0f / 3.0f, quad));
     return rmul(rmul(2.0f, w), radd(m.drb, con));
 }
 
+// The coefficient of c.j* in the bounce-back rule of link i = opp(k).
+__device__ __forceinline__ float bounce_factor(int k, float fac) {
+    return -rmul(fac, rmul(6.0f, k <= 4 ? (1.0f / 9.0f) : (1.0f / 36.0f)));
+}
+
 // Eq. (bbnoncon) for link i = opp(k) given j*; kappa = 0, 1 + kappa = 1 (q = 1/2)
 // give Eq. (bbcon).
 __device__ __forceinline__ float bounce_back(int k, float kap, float fac, float gk, float gi,
                                              float gy_i, float jsx, float jsy) {
-    const int i = k <= 4 ? (k + 1) % 4 + 1 : (k - 3) % 4 + 5;
-    const float w = (i <= 4) ? (1.0f / 9.0f) : (1.0f / 36.0f);
-    const float cix = (float)(-lane_cx(k)), ciy = (float)(-lane_cy(k));
+    const float cix = link_cx(k), ciy = link_cy(k);
     const float cj = rfma(cix, jsx, rmul(ciy, jsy));
-    return rfma(-rmul(fac, rmul(6.0f, w)), cj, rfma(kap, rsub(gy_i, gk), gi));
+    return rfma(bounce_factor(k, fac), cj, rfma(kap, rsub(gy_i, gk), gi));
 }
 
 // Eq. (abbnoncon) for link i = opp(k) given its wall equilibrium term.
@@ -533,12 +555,71 @@ __device__ __forceinline__ float anti_bounce_back(float kap, float fac, float gk
     return rfma(fac, eq, rfma(-kap, radd(gy_i, gk), -gi));
 }
 
+// What a cut link's rule needs that does not depend on the populations: from
+// the link record and the boundary data at time tb.  A path that steps a link
+// several times keeps it for as long as the data do not change.
+struct LinkRule {
+    float q, kap, fac;    // wall distance, kappa, 1 + kappa (Dirichlet: bounce_factor)
+    float t0, t1;         // Neumann: tangent
+    float c0, c1, c2;     // Neumann: WallData, or sigma* at a corner; Dirichlet: c0 = c.j*
+};
+
+__device__ __forceinline__ LinkRule link_rule(int k, bool miss, bool dirich, bool corner,
+                                              const BLink &lk, const BCDev *__restrict__ bcs,
+                                              float tb, const Lattice &L) {
+    LinkRule r;
+    r.q = miss ? 0.5f : lk.q;
+    link_kappa(r.q, r.kap, r.fac);
+    if (dirich) {
+        float jsx, jsy;
+        dirichlet_momentum(lk, bcs, tb, L, jsx, jsy);
+        r.fac = bounce_factor(k, r.fac);
+        r.c0 = rfma(link_cx(k), jsx, rmul(link_cy(k), jsy));
+        r.t0 = r.t1 = r.c1 = r.c2 = 0.0f;
+    } else if (corner) {
+        float tax, tay, tbx, tby;
+        traction(bcs[lk.bc], lk.n0, 0.0f, tb, tax, tay);
+        traction(bcs[lk.bc2], 0.0f, lk.n1, tb, tbx, tby);
+        r.t0 = r.t1 = 0.0f;
+        r.c0 = rmul(tax, lk.n0);
+        r.c1 = rmul(tby, lk.n1);
+        r.c2 = rmul(0.5f, rfma(tay, lk.n0, rmul(tbx, lk.n1)));
+    } else {
+        const WallFrame w = wall_frame(lk, bcs, tb);
+        const WallData d = wall_data(w);
+        r.t0 = w.t0;
+        r.t1 = w.t1;
+        r.c0 = d.cxx;
+        r.c1 = d.cyy;
+        r.c2 = d.cxy;
+    }
+    return r;
+}
+
 // f_k(x, t) arriving through the cut link i = opp(k) of a boundary node:
 // Eq. (bbnoncon) for a Dirichlet link, Eq. (abbnoncon) for a Neumann one (both
 // reduce to Eqs. bbcon/abbcon at q = 1/2).  gk, gi: f_k^col(x), f_i^col(x) at
-// t-1; gy_i: f_i^col(x - c_i) (0 if the upstream node is unusable, `miss`);
-// dr_x, p**_x: density deviation and P of f^col(x); my_*: the same moments at
+// t-1; gy_i: f_i^col(x - c_i) (0 if the upstream node is unusable); dr_x,
+// p**_x: density deviation and P of f^col(x); my_*: the same moments at
 // x - c_i, used when the Neumann wall values are extrapolated (`neu_ex`).
+__device__ __forceinline__ float link_value(int k, const LinkRule &r, bool dirich, bool corner,
+                                            bool neu_ex, float gk, float gi, float gy_i, float dr_x,
+                                            float pxx_x, float pyy_x, float pxy_x, float my_dr,
+                                            float my_xx, float my_yy, float my_xy,
+                                            const Lattice &L) {
+    // both rules, selected at the end: the links of a warp need not agree
+    const float bb = rfma(r.fac, r.c0, rfma(r.kap, rsub(gy_i, gk), gi));
+    const WallState st = wall_state(neu_ex, r.q, dr_x, pxx_x, pyy_x, pxy_x, my_dr, my_xx, my_yy,
+                                    my_xy, L);
+    float sxx, syy, sxy;  // sigma* (Eq. trafocauchy)
+    wall_sigma(r.t0, r.t1, WallData{r.c0, r.c1, r.c2}, st, sxx, syy, sxy);
+    sxx = corner ? r.c0 : sxx;
+    syy = corner ? r.c1 : syy;
+    sxy = corner ? r.c2 : sxy;
+    const float eq = wall_equilibrium(k, wall_moments(st.drb, sxx, syy, sxy, L));
+    return dirich ? bb : anti_bounce_back(r.kap, r.fac, gk, gi, gy_i, eq);
+}
+
 __device__ __forceinline__ float cut_link_value(int k, bool miss, bool dirich, bool corner,
                                                 bool neu_ex, const BLink &lk, float gk, float gi,
                                                 float gy_i, float dr_x, float pxx_x, float pyy_x,
@@ -546,29 +627,8 @@ __device__ __forceinline__ float cut_link_value(int k, bool miss, bool dirich, b
                                                 float my_yy, float my_xy,
                                                 const BCDev *__restrict__ bcs, float tb,
                                                 const Lattice &L) {
-    const float q = miss ? 0.5f : lk.q;
-    float kap, fac;
-    link_kappa(q, kap, fac);
-    if (dirich) {
-        float jsx, jsy;
-        dirichlet_momentum(lk, bcs, tb, L, jsx, jsy);
-        return bounce_back(k, kap, fac, gk, gi, gy_i, jsx, jsy);
-    }
-    const WallState st = wall_state(neu_ex, q, dr_x, pxx_x, pyy_x, pxy_x, my_dr, my_xx, my_yy,
-                                    my_xy, L);
-    float sxx, syy, sxy;  // sigma* (Eq. trafocauchy)
-    if (corner) {
-        float tax, tay, tbx, tby;
-        traction(bcs[lk.bc], lk.n0, 0.0f, tb, tax, tay);
-        traction(bcs[lk.bc2], 0.0f, lk.n1, tb, tbx, tby);
-        sxx = rmul(tax, lk.n0);
-        syy = rmul(tby, lk.n1);
-        sxy = rmul(0.5f, rfma(tay, lk.n0, rmul(tbx, lk.n1)));
-    } else {
-        wall_sigma(wall_frame(lk, bcs, tb), st, sxx, syy, sxy);
-    }
-    const float eq = wall_equilibrium(k, wall_moments(st.drb, sxx, syy, sxy, L));
-    return anti_bounce_back(kap, fac, gk, gi, gy_i, eq);
+    return link_value(k, link_rule(k, miss, dirich, corner, lk, bcs, tb, L), dirich, corner, neu_ex,
+                      gk, gi, gy_i, dr_x, pxx_x, pyy_x, pxy_x, my_dr, my_xx, my_yy, my_xy, L);
 }
 
 // Populations f(x, t) of a boundary node: pulled where the link is intact,

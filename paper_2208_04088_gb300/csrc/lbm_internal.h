@@ -276,6 +276,78 @@ cudaError_t launch_wave_batch(const WaveInst *insts, const int4 *regions, const 
 cudaError_t launch_wave(const Lattice &L, const DevState &S, const WaveMaps &m, int cur, int toff,
                         cudaStream_t s, long long *cycles = nullptr);
 
+// Register-tile stepping (kernels in lbm_tile.cu, tables in lbm_plan.cpp).  A
+// tile shape is the threads to a row (two columns each) and the rows to a
+// thread; kTileThreads threads make a block.
+constexpr int kTileThreads = 512;
+constexpr int kTileHalo = 8;      // kWaveK steps of one node, kWaveGradK of two
+static_assert(kTileHalo >= kWaveK && kTileHalo >= 2 * kWaveGradK, "tile halo");
+struct TileShape {
+    int lpr, rows;
+    constexpr int w() const { return 2 * lpr; }
+    constexpr int h() const { return kTileThreads / lpr * rows; }
+    // nodes of a tile that boundary rules may read: every node of the smallest
+    // tile, as many as the shared memory leaves room for in the others
+    constexpr int slots() const { return w() * h() <= 1024 ? 1024 : 512; }
+};
+constexpr TileShape kTileShapes[] = {{16, 1}, {32, 2}, {32, 3}, {32, 4}};
+constexpr int kTileShapeCount = 4;
+static_assert(kTileShapes[0].w() * kTileShapes[0].h() <= kTileShapes[0].slots(),
+              "the smallest tile can publish every node");
+
+struct TileRec {
+    int32_t x0, y0;          // lattice node of ring node (0, 0)
+    int16_t c0, c1, r0, r1;  // core columns [c0, c1) and rows [r0, r1) of the ring
+    int32_t pub0, link0;     // first entry of the published-node and link tables
+    uint16_t npub, nlink;
+    int32_t inst;            // instance of a batch
+};
+static_assert(sizeof(TileRec) == 32, "TileRec layout");
+
+enum : uint8_t {
+    kLinkMiss = 1, kLinkDirichlet = 2, kLinkCorner = 4,
+    kLinkExtrapolate = 8,  // Neumann wall values extrapolated from the upstream node
+    kLinkUpstream = 16     // the rule reads the upstream node (its slot is valid)
+};
+// One cut link of a tile; own, up: slots of its node and of the upstream node.
+struct alignas(8) TileLink {
+    uint16_t own, up, bc, bc2;
+    float q, n0, n1;
+    uint8_t dir, flags, pad[2];
+};
+static_assert(sizeof(TileLink) == 24, "TileLink layout");
+
+// Host tables of a lattice cut into tiles: published nodes as column |
+// row << 8 | cut mask << 16 (bit i - 1 for direction i), slots in table order.
+struct TilePlan {
+    int shape = -1;  // index into kTileShapes, -1: none
+    std::vector<TileRec> tiles;
+    std::vector<uint32_t> pubs;
+    std::vector<TileLink> links;
+};
+// Cuts the lattice into tiles of a shape; false if a tile would have to
+// publish more nodes than its shape holds (never with shape 0).
+bool tile_plan(const Tables &t, bool wall_node, int shape, TilePlan *p);
+// The shape with the smallest modelled time per launch, and its plan;
+// p->shape is -1 where one step per launch is modelled to be faster.
+void tile_choose(const Tables &t, bool grad, bool wall_node, int sms, TilePlan *p);
+
+// Device side of a plan (tables owned by the handle, outside its workspace).
+struct TileDev {
+    CUtensorMap map[2];  // the population buffers, box of one tile
+    int shape = -1, ntiles = 0;
+    const TileRec *tiles = nullptr;
+    const uint32_t *pubs = nullptr;
+    const TileLink *links = nullptr;
+    void *mem = nullptr;
+};
+bool tile_supported();
+cudaError_t tile_prepare(const Lattice &L, const DevState &S, TileDev *T);
+// nsteps (1 .. kWaveK, or kWaveGradK when lambda != mu) steps from buffer
+// `cur` into cur ^ 1.
+cudaError_t launch_tile(const Lattice &L, const DevState &S, const TileDev &T, int cur, int toff,
+                        int nsteps, cudaStream_t s);
+
 }  // namespace lbm
 
 // One solver instance (the object behind lbm_handle).
@@ -309,5 +381,6 @@ struct lbm_solver {
     // temporal blocking: steps per launch (1: one-step kernels) and its tables
     int block = 1;
     lbm::WaveMaps wave;
+    lbm::TileDev tile;  // register tiles, when in use (shape >= 0)
 };
 

@@ -4,8 +4,11 @@
 // cache of measured plans.  The kernels are in lbm_wave.cu.
 #include <algorithm>
 #include <cstdint>
+#include <cstring>
+#include <functional>
 #include <map>
 #include <mutex>
+#include <queue>
 #include <tuple>
 #include <vector>
 
@@ -353,6 +356,211 @@ cudaError_t wave_calibrate(const Tables &t, const Lattice &L, const DevState &S,
     // pageable source: the copy is staged before the call returns
     return cudaMemcpyAsync(S.wave_tab, best.data(), best.size() * sizeof(int4),
                            cudaMemcpyHostToDevice, s);
+}
+
+// ---------------------------------------------------------------------------
+// Register tiles (lbm_tile.cu).
+
+namespace {
+
+// Rings of `w` nodes along an axis of n: ring k starts at k (w - 2 kTileHalo)
+// and owns what neither neighbour does; the ends need no halo, so the box
+// edges belong to the first and last ring's core.
+int ring_count(int n, int w) {
+    return n <= w ? 1 : (n - 2 * kTileHalo + w - 2 * kTileHalo - 1) / (w - 2 * kTileHalo);
+}
+
+// use(k) for every ring k = ty ntx + tx that holds the boundary node.
+template <class Use> void for_rings(const BNode &b, int W, int H, int ntx, int nty, Use use) {
+    const int sx = W - 2 * kTileHalo, sy = H - 2 * kTileHalo;
+    const int tx1 = std::min(ntx - 1, b.x / sx), ty1 = std::min(nty - 1, b.y / sy);
+    for (int ty = ty1; ty >= 0 && b.y < ty * sy + H; --ty)
+        for (int tx = tx1; tx >= 0 && b.x < tx * sx + W; --tx) use((size_t)ty * ntx + tx);
+}
+
+}  // namespace
+
+bool tile_plan(const Tables &t, bool wall_node, int shape, TilePlan *p) {
+    const TileShape sh = kTileShapes[shape];
+    const int W = sh.w(), H = sh.h(), sx = W - 2 * kTileHalo, sy = H - 2 * kTileHalo;
+    const int ntx = ring_count(t.nx, W), nty = ring_count(t.ny, H);
+    p->shape = shape;
+    p->tiles.clear();
+    p->pubs.clear();
+    p->links.clear();
+    // boundary nodes seen by each ring: seen[first[k] .. first[k + 1])
+    std::vector<int32_t> first((size_t)ntx * nty + 1, 0), seen;
+    for (const BNode &b : t.bnodes)
+        for_rings(b, W, H, ntx, nty, [&](size_t k) { ++first[k + 1]; });
+    for (size_t k = 1; k < first.size(); ++k) first[k] += first[k - 1];
+    seen.resize((size_t)first.back());
+    {
+        std::vector<int32_t> at(first.begin(), first.end() - 1);
+        for (size_t g = 0; g < t.bnodes.size(); ++g)
+            for_rings(t.bnodes[g], W, H, ntx, nty, [&](size_t k) { seen[(size_t)at[k]++] = (int32_t)g; });
+    }
+    p->tiles.reserve((size_t)ntx * nty);
+    p->pubs.reserve(2 * seen.size());
+    p->links.reserve(4 * seen.size());
+    std::vector<int32_t> slot((size_t)W * H, -1);
+    for (int ty = 0; ty < nty; ++ty)
+        for (int tx = 0; tx < ntx; ++tx) {
+            TileRec r;
+            std::memset(&r, 0, sizeof r);
+            r.x0 = tx * sx;
+            r.y0 = ty * sy;
+            r.c0 = tx == 0 ? 0 : kTileHalo;
+            r.r0 = ty == 0 ? 0 : kTileHalo;
+            r.c1 = (int16_t)(tx == ntx - 1 ? t.nx - r.x0 : W - kTileHalo);
+            r.r1 = (int16_t)(ty == nty - 1 ? t.ny - r.y0 : H - kTileHalo);
+            r.pub0 = (int32_t)p->pubs.size();
+            r.link0 = (int32_t)p->links.size();
+            const size_t tile = (size_t)ty * ntx + tx;
+            if (first[tile] == first[tile + 1]) {
+                // without boundary nodes a tile holds material or void alone
+                const int x = r.x0 + r.c0, y = r.y0 + r.r0;
+                if (t.cls[(size_t)y * t.pitch + x] == kVoid && !(tx == ntx - 1 && ty == nty - 1 &&
+                                                                p->tiles.empty()))
+                    continue;
+                p->tiles.push_back(r);
+                continue;
+            }
+            int count = 0;
+            auto publish = [&](int c, int row) {
+                int32_t &s = slot[(size_t)row * W + c];
+                if (s < 0) {
+                    s = count++;
+                    p->pubs.push_back((uint32_t)c | (uint32_t)row << 8);
+                }
+                return s;
+            };
+            for (int32_t q = first[tile]; q < first[tile + 1]; ++q) {
+                const int32_t gi = seen[(size_t)q];
+                const BNode &b = t.bnodes[gi];
+                const int c = b.x - r.x0, row = b.y - r.y0;
+                // the ring's outermost nodes beside a neighbouring tile are
+                // never computed
+                if ((tx > 0 && c < 1) || (tx < ntx - 1 && c > W - 2) || (ty > 0 && row < 1) ||
+                    (ty < nty - 1 && row > H - 2))
+                    continue;
+                const int own = publish(c, row);
+                p->pubs[r.pub0 + own] |= (uint32_t)((b.cut >> 1) & 0xffu) << 16;
+                for (int i = 1; i < kQ; ++i) {
+                    const uint32_t bit = 1u << i;
+                    if (!(b.cut & bit)) continue;
+                    const BLink &lk = t.blinks[(size_t)gi * 8 + i - 1];
+                    TileLink e;
+                    std::memset(&e, 0, sizeof e);
+                    const bool miss = b.miss & bit, dir = b.dirich & bit;
+                    e.own = (uint16_t)own;
+                    e.dir = (uint8_t)i;
+                    e.q = lk.q;
+                    e.n0 = lk.n0;
+                    e.n1 = lk.n1;
+                    e.bc = lk.bc;
+                    e.bc2 = lk.bc2;
+                    if (miss) e.flags |= kLinkMiss;
+                    if (dir) e.flags |= kLinkDirichlet;
+                    if (b.corner & bit) e.flags |= kLinkCorner;
+                    if (!miss && !dir && !wall_node) e.flags |= kLinkExtrapolate;
+                    if (!miss && (lk.q != 0.5f || (e.flags & kLinkExtrapolate))) {
+                        e.flags |= kLinkUpstream;
+                        e.up = (uint16_t)publish(c - kCx[i], row - kCy[i]);
+                    }
+                    p->links.push_back(e);
+                }
+            }
+            for (size_t k = r.pub0; k < p->pubs.size(); ++k)
+                slot[(size_t)((p->pubs[k] >> 8) & 0xffu) * W + (p->pubs[k] & 0xffu)] = -1;
+            if (count > sh.slots()) return false;
+            r.npub = (uint16_t)count;
+            r.nlink = (uint16_t)(p->links.size() - r.link0);
+            p->tiles.push_back(r);
+        }
+    // tiles with links first: they take longest
+    std::stable_sort(p->tiles.begin(), p->tiles.end(),
+                     [](const TileRec &a, const TileRec &b) { return a.nlink > b.nlink; });
+    return true;
+}
+
+namespace {
+
+// Modelled time (us) of one launch with a shape: every tile costs a fixed part
+// (copy in, store) and per step a part for its nodes, one for having boundary
+// rules at all (two more barriers and a link's dependent chain) and one per
+// link; the tiles, those with links first, are taken by `sms` SMs, one each.
+// Constants per shape from GB300 timings of lattices of 64^2 to 2048^2 nodes (8 steps: 17 us for a
+// wave of 32 x 32 tiles with links, 9 us without; 24 us for 64 x 64 without).
+double tile_time(const Tables &t, int shape, bool grad, int sms) {
+    static const double kFixed[kTileShapeCount] = {4.0, 5.0, 6.0, 6.5};
+    static const double kNodes[kTileShapeCount] = {0.7, 1.2, 1.6, 1.75};
+    static const double kRules[kTileShapeCount] = {0.7, 1.3, 1.6, 1.9};
+    const double kLink = 0.0008;
+    const int W = kTileShapes[shape].w(), H = kTileShapes[shape].h();
+    const int ntx = ring_count(t.nx, W), nty = ring_count(t.ny, H);
+    const int steps = grad ? kWaveGradK : kWaveK;
+    std::vector<int32_t> links((size_t)ntx * nty, 0);
+    for (const BNode &b : t.bnodes) {
+        const int n = __builtin_popcount(b.cut);
+        for_rings(b, W, H, ntx, nty, [&](size_t k) { links[k] += n; });
+    }
+    const double plain = kFixed[shape] + steps * (grad ? 1.3 : 1.0) * kNodes[shape];
+    // the tiles with links go first, in order; the others fill up evenly
+    std::priority_queue<double, std::vector<double>, std::greater<double>> sm;
+    for (int k = 0; k < sms; ++k) sm.push(0.0);
+    double end = 0.0, total = 0.0;
+    size_t without = 0;
+    for (const int32_t n : links) {
+        if (!n) {
+            ++without;
+            continue;
+        }
+        const double c = plain + steps * ((grad ? 1.5 : 1.0) * kRules[shape] + kLink * n);
+        const double at = sm.top() + c;
+        sm.pop();
+        sm.push(at);
+        end = std::max(end, at);
+        total += c;
+    }
+    // the others one by one while they are few, by their sum while they are many
+    if (without <= (size_t)4 * sms) {
+        for (; without; --without) {
+            const double at = sm.top() + plain;
+            sm.pop();
+            sm.push(at);
+            end = std::max(end, at);
+        }
+        return end;
+    }
+    return std::max(end, (total + (double)without * plain) / sms + 0.5 * plain);
+}
+
+}  // namespace
+
+void tile_choose(const Tables &t, bool grad, bool wall_node, int sms, TilePlan *p) {
+    // One step per launch: bound by launches (two kernels beside each other,
+    // or three in a row with the density pass), by the bytes of a step, and by
+    // the eight lanes of every boundary node.  A lattice with walls everywhere
+    // (a porous solid) stays with it: only the smallest tiles hold its nodes.
+    const double nodes = (double)t.nx * t.ny;
+    const double step = grad ? std::max(14.0, 2.0 + 21.2e-6 * nodes)
+                             : std::max(4.2, 1.0 + (nodes < 1e6 ? 11.6e-6 : 15.7e-6) * nodes);
+    const double limit =
+        (grad ? kWaveGradK : kWaveK) * (step + 1.2e-4 * (double)t.bnodes.size());
+    std::vector<std::pair<double, int>> order;
+    // from the largest tile down; once a shape fills the SMs several times
+    // over, smaller tiles only add halo
+    for (int s = kTileShapeCount - 1; s >= 0; --s) {
+        order.emplace_back(tile_time(t, s, grad, sms), s);
+        if ((size_t)ring_count(t.nx, kTileShapes[s].w()) * ring_count(t.ny, kTileShapes[s].h()) >
+            (size_t)8 * sms)
+            break;
+    }
+    if (order.back().second > 0) order.emplace_back(tile_time(t, 0, grad, sms), 0);
+    std::stable_sort(order.begin(), order.end());
+    for (const auto &o : order)
+        if (o.first <= limit && tile_plan(t, wall_node, o.second, p)) return;
+    p->shape = -1;
 }
 
 }  // namespace lbm
