@@ -326,8 +326,8 @@ const char *lbm_last_error(void);
  * node; the simple nodes of box edges and crack faces one lane each), running
  * the same per-node code as lbm_step, so every instance's fields are
  * bit-identical to the same instance stepped alone.  FP32 instances of at
- * least 128 columns are stepped instead by the temporally blocked kernel, 8
- * steps per launch over all of them.  Steps replay a captured CUDA graph.
+ * least 128 columns are stepped instead in register tiles, 8 steps per launch
+ * over all of them.  Steps replay a captured CUDA graph.
  * ------------------------------------------------------------------------ */
 typedef struct lbm_engine *lbm_batch;
 typedef struct lbm_engine *lbm_server;
@@ -349,22 +349,21 @@ typedef struct {
     uint64_t device_bytes;   /* arena bytes in use */
     int64_t kernel_launches;
     lbm_launch_shape shape;
-    int32_t blocked_instances; /* instances stepped by the temporally blocked kernel */
+    int32_t blocked_instances; /* instances stepped several steps per launch */
     int32_t pad;
 } lbm_batch_stats;
 
 /* Create a batch of `count` instances (host descriptors as for lbm_create,
  * every one with lambda = mu and the same storage), all at rest at t = 0.
- * FP32 instances with two population buffers and nx >= 128 are stepped by the
- * temporally blocked kernel: one persistent launch per LBM_TIME_BLOCK steps
- * over the strip segments of all of them (segments of about 768 rows, the
- * longest first, taken by the blocks from a counter).  The other instances
- * are stepped one step per launch by the batched interior and boundary
- * kernels.  time_block of the descriptors is not used; each instance keeps
- * the streaming form its descriptor asks for, and in-place instances take
- * less of the arena.  Either way every instance's fields are bit-identical
- * to the instance stepped alone.  Device memory: one arena sized for all
- * instances.  Synchronous. */
+ * FP32 instances with two population buffers and nx >= 128 are stepped in
+ * register tiles: one launch per LBM_TIME_BLOCK steps over the tiles of all of
+ * them.  The other instances are stepped one step per launch by the batched
+ * interior and boundary kernels.  time_block of the descriptors is not used;
+ * each instance keeps the streaming form its descriptor asks for, and in-place
+ * instances take less of the arena.  Either way every instance's fields are
+ * bit-identical to the instance stepped alone.  Device memory: one arena sized
+ * for all instances, and the work tables (of the tiles: about 100 bytes per
+ * boundary node).  Synchronous. */
 lbm_status lbm_batch_create(const lbm_desc *descs, int32_t count, void *stream, lbm_batch *out);
 /* Advance every instance by nsteps (asynchronous). */
 lbm_status lbm_batch_step(lbm_batch b, int64_t nsteps);

@@ -12,10 +12,9 @@
 // valid while instances come and go.
 //
 // In the lockstep batch, FP32 instances with two population buffers and at
-// least kWaveC columns are stepped by the temporally blocked kernel instead:
-// one persistent launch per kWaveK steps over the strip segments (regions) of
-// all of them, longest first, each block taking the next region from a
-// counter.  Its per-node arithmetic is that of the one-step kernels too.
+// least kWaveC columns are stepped in register tiles instead (lbm_tile.cu): one
+// launch per kWaveK steps over the tiles of all of them, those with boundary
+// rules first.  The per-node arithmetic is that of the one-step kernels too.
 #include <algorithm>
 #include <chrono>
 #include <climits>
@@ -48,7 +47,7 @@ struct InstDev {
     int64_t *time;   // completed steps (the instance's own clock)
     int64_t target;  // the instance stops stepping at this time
     int32_t tiles_x;
-    int32_t blocked;  // stepped by the temporally blocked batch kernel
+    int32_t blocked;  // stepped in register tiles
 };
 
 // Sizes of the work tables and the dynamic-schedule counters (device memory).
@@ -360,8 +359,7 @@ struct DescCopy {
 
 struct Instance {
     int64_t id = -1;
-    bool blocked = false;  // stepped by the blocked batch kernel
-    int plan_blocks = 0;   // its regions (strip segments)
+    bool blocked = false;  // stepped in register tiles
     lbm_solver *h = nullptr;
     uint64_t off = 0, bytes = 0;
     int64_t steps = 0;   // requested steps
@@ -427,11 +425,10 @@ struct lbm_engine {
     int sms = 0;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // by the blocked instances' buffer
     bool graph_in_place = false;  // the captured graph orders the boundary kernel first
-    // instances stepped by the blocked kernel: their records and regions
-    WaveInst *d_winst = nullptr;
-    int4 *d_regions = nullptr;
-    int32_t *d_region_inst = nullptr, *d_wcounter = nullptr;
-    int cap_winst = 0, cap_regions = 0, nregions = 0, nblocked = 0;
+    // instances stepped in tiles: their records and tables (one allocation)
+    TileBatch tile;
+    void *d_tile = nullptr;
+    int nblocked = 0;
     int wcur = 0;  // the buffer that holds their populations
     // pinned staging of the table uploads (reused once the last upload is done)
     char *h_stage = nullptr;
@@ -491,87 +488,89 @@ lbm_status ensure_capacity(lbm_engine *E, int ninst, int64_t ntiles, int64_t nbn
     return LBM_OK;
 }
 
-// Regions of the blocked instances: per instance, the strip segments of a
-// plan for plan_blocks blocks; all of them ordered by the planner's modelled
-// cost (row sweeps, boundary updates included), the most expensive first, so
-// that the blocks that take them from the counter end close together.
-lbm_status rebuild_wave_tables(lbm_engine *E) {
-    bool any = E->nblocked > 0;
-    for (const Instance &I : E->inst) any = any || I.blocked;
-    if (!any) return LBM_OK;
-    std::vector<WaveInst> wi;
-    std::vector<std::pair<int, int4>> reg;  // (record, region)
-    std::vector<double> cost;
-    for (size_t i = 0; i < E->inst.size(); ++i) {
-        const Instance &I = E->inst[i];
-        if (!I.blocked) continue;
-        const lbm_solver *h = I.h;
-        WaveInst w;
-        std::memset(&w, 0, sizeof w);
-        w.tf[0] = h->wave.f[0];
-        w.tf[1] = h->wave.f[1];
-        w.tnw = h->wave.nw;
-        w.tu = h->wave.u;
-        w.f[0] = static_cast<float *>(h->S.f[0]);
-        w.f[1] = static_cast<float *>(h->S.f[1]);
-        w.uc = static_cast<float4 *>(h->S.ucomp);
-        w.blinks = h->S.blinks;
-        w.bcs = h->S.bcs;
-        w.time = h->S.time;
-        w.status = h->S.status;
-        w.L = h->L;
-        const std::vector<int4> plan = wave_plan(h->tab, I.plan_blocks);
-        const std::vector<double> c = wave_plan_costs(h->tab, plan);
-        for (size_t r = 0; r < plan.size(); ++r) {
-            reg.emplace_back((int)wi.size(), plan[r]);
-            cost.push_back(c[r]);
+// Tables of the instances stepped in register tiles, built once: a lockstep
+// batch keeps its instances.  One tile shape for all of them, the one with the
+// smallest modelled time summed over the batch (its tiles fill the SMs many
+// times over, so sums count, not the longest tile); the tiles with the most
+// cut links first, so that the last ones to end are the short ones.
+lbm_status build_tile_tables(lbm_engine *E) {
+    if (E->d_tile) return LBM_OK;
+    std::vector<const lbm_solver *> who;
+    for (const Instance &I : E->inst)
+        if (I.blocked) who.push_back(I.h);
+    if (who.empty()) return LBM_OK;
+    std::vector<std::pair<double, int>> order;
+    for (int s = 0; s < kTileShapeCount; ++s) {
+        double sum = 0.0;
+        for (const lbm_solver *h : who) sum += tile_time(h->tab, s, false, 1);
+        order.emplace_back(sum, s);
+    }
+    std::sort(order.begin(), order.end());
+    std::vector<TileInst> inst;
+    TilePlan all;
+    for (const auto &o : order) {
+        inst.clear();
+        all = TilePlan();
+        all.shape = o.second;
+        bool ok = true;
+        for (size_t i = 0; i < who.size() && ok; ++i) {
+            const lbm_solver *h = who[i];
+            TileInst w;
+            std::memset(&w, 0, sizeof w);
+            if (!tile_maps(h->L, h->S, all.shape, w.map))
+                return fail_cuda(cudaErrorInvalidValue, "batch: tensor maps");
+            w.f[0] = static_cast<float *>(h->S.f[0]);
+            w.f[1] = static_cast<float *>(h->S.f[1]);
+            w.uc = static_cast<float4 *>(h->S.ucomp);
+            w.cls = h->S.cls;
+            w.bcs = h->S.bcs;
+            w.time = h->S.time;
+            w.status = h->S.status;
+            w.L = h->L;
+            TilePlan p;
+            ok = tile_plan(h->tab, h->L.wall_node != 0, all.shape, &p);
+            for (TileRec r : p.tiles) {
+                r.inst = (int32_t)i;
+                r.pub0 += (int32_t)all.pubs.size();
+                r.link0 += (int32_t)all.links.size();
+                all.tiles.push_back(r);
+            }
+            all.pubs.insert(all.pubs.end(), p.pubs.begin(), p.pubs.end());
+            all.links.insert(all.links.end(), p.links.begin(), p.links.end());
+            inst.push_back(w);
         }
-        wi.push_back(w);
+        if (ok) break;  // the smallest tiles always are
     }
-    std::vector<size_t> order(reg.size());
-    for (size_t r = 0; r < order.size(); ++r) order[r] = r;
-    std::stable_sort(order.begin(), order.end(),
-                     [&cost](size_t a, size_t b) { return cost[a] > cost[b]; });
-    std::vector<int4> regions(reg.size());
-    std::vector<int32_t> rinst(reg.size());
-    for (size_t r = 0; r < reg.size(); ++r) {
-        regions[r] = reg[order[r]].second;
-        rinst[r] = reg[order[r]].first;
-    }
-    cudaError_t e = cudaSuccess;
-    if ((int)wi.size() > E->cap_winst) {
-        if (E->d_winst) cudaFree(E->d_winst);
-        E->cap_winst = std::max((int)wi.size(), 2 * E->cap_winst);
-        e = cudaMalloc(&E->d_winst, sizeof(WaveInst) * E->cap_winst);
-        drop_graphs(E);
-    }
-    if (e == cudaSuccess && (int)regions.size() > E->cap_regions) {
-        if (E->d_regions) cudaFree(E->d_regions);
-        if (E->d_region_inst) cudaFree(E->d_region_inst);
-        E->cap_regions = std::max((int)regions.size(), 2 * E->cap_regions);
-        e = cudaMalloc(&E->d_regions, sizeof(int4) * E->cap_regions);
-        if (e == cudaSuccess) e = cudaMalloc(&E->d_region_inst, sizeof(int32_t) * E->cap_regions);
-        drop_graphs(E);
-    }
-    if (e == cudaSuccess && !E->d_wcounter) e = cudaMalloc(&E->d_wcounter, sizeof(int32_t));
+    std::stable_sort(all.tiles.begin(), all.tiles.end(),
+                     [](const TileRec &a, const TileRec &b) { return a.nlink > b.nlink; });
+    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+    const size_t bi = up(sizeof(TileInst) * inst.size()), bt = up(sizeof(TileRec) * all.tiles.size());
+    const size_t bp = up(sizeof(uint32_t) * all.pubs.size()), bl = sizeof(TileLink) * all.links.size();
+    cudaError_t e = cudaMalloc(&E->d_tile, bi + bt + bp + bl);
+    if (e != cudaSuccess) return fail_cuda(e, "batch: tile tables");
+    char *m = static_cast<char *>(E->d_tile);
+    E->tile.shape = all.shape;
+    E->tile.insts = reinterpret_cast<const TileInst *>(m);
+    E->tile.tiles = reinterpret_cast<const TileRec *>(m + bi);
+    E->tile.pubs = reinterpret_cast<const uint32_t *>(m + bi + bt);
+    E->tile.links = reinterpret_cast<const TileLink *>(m + bi + bt + bp);
     // sets the kernel's shared-memory limit (outside any capture); launches nothing
-    if (e == cudaSuccess && !wi.empty())
-        e = launch_wave_batch(nullptr, nullptr, nullptr, 0, nullptr, 0, 0, E->sms, E->stream);
-    if (e != cudaSuccess) return fail_cuda(e, "batch: blocked tables");
-    if ((int)regions.size() != E->nregions || (int)wi.size() != E->nblocked) drop_graphs(E);
-    E->nregions = (int)regions.size();
-    E->nblocked = (int)wi.size();
-    if (!wi.empty())
-        e = cudaMemcpyAsync(E->d_winst, wi.data(), sizeof(WaveInst) * wi.size(),
+    e = launch_tile_batch(E->tile, 0, 0, 0, E->stream);
+    E->tile.ntiles = (int)all.tiles.size();
+    E->nblocked = (int)inst.size();
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(m, inst.data(), sizeof(TileInst) * inst.size(), cudaMemcpyHostToDevice,
+                            E->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(m + bi, all.tiles.data(), sizeof(TileRec) * all.tiles.size(),
                             cudaMemcpyHostToDevice, E->stream);
-    if (e == cudaSuccess && !regions.empty())
-        e = cudaMemcpyAsync(E->d_regions, regions.data(), sizeof(int4) * regions.size(),
+    if (e == cudaSuccess && !all.pubs.empty())
+        e = cudaMemcpyAsync(m + bi + bt, all.pubs.data(), sizeof(uint32_t) * all.pubs.size(),
                             cudaMemcpyHostToDevice, E->stream);
-    if (e == cudaSuccess && !rinst.empty())
-        e = cudaMemcpyAsync(E->d_region_inst, rinst.data(), sizeof(int32_t) * rinst.size(),
-                            cudaMemcpyHostToDevice, E->stream);
+    if (e == cudaSuccess && !all.links.empty())
+        e = cudaMemcpyAsync(m + bi + bt + bp, all.links.data(), bl, cudaMemcpyHostToDevice, E->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(E->stream);  // the host vectors die here
-    if (e != cudaSuccess) return fail_cuda(e, "batch: blocked tables upload");
+    if (e != cudaSuccess) return fail_cuda(e, "batch: tile tables upload");
     return LBM_OK;
 }
 
@@ -621,7 +620,7 @@ lbm_status rebuild_tables(lbm_engine *E) {
     if (E->shape.dynamic >= 2 && (int64_t)tiles.size() != E->ntiles) {
         drop_graphs(E);  // one block per tile: the captured grid must match the table
     }
-    lbm_status wst = rebuild_wave_tables(E);
+    lbm_status wst = build_tile_tables(E);
     if (wst != LBM_OK) return wst;
     E->ntiles = (int64_t)tiles.size();
     BatchCounts c;
@@ -764,26 +763,21 @@ cudaError_t launch_batch_step(lbm_engine *E, cudaStream_t s_main, cudaStream_t s
     }
 }
 
-// kChunk steps of the instances stepped by the blocked kernel: kChunk/kWaveK
-// launches from buffer `wcur` (an even number, so they end in it), then their
-// clocks.  They read the clocks at the start of the chunk (toff = the launch's
-// first step within it).
-static_assert(kChunk % (2 * kWaveK) == 0, "blocked launches per chunk");
+// n steps of the instances stepped in tiles, from buffer `cur`, then their
+// clocks; the launches read the clocks as they were (toff = a launch's first
+// step).  Returns in *cur the buffer they end in.
+static_assert(kChunk % (2 * kWaveK) == 0, "a chunk ends in the buffer it starts from");
 
-cudaError_t launch_blocked_chunk(lbm_engine *E, cudaStream_t s) {
+cudaError_t launch_blocked(lbm_engine *E, int64_t n, int *cur, cudaStream_t s) {
     if (E->nblocked == 0) return cudaSuccess;
     cudaError_t e = cudaSuccess;
-    int cur = E->wcur;
-    for (int toff = 0; toff < kChunk && e == cudaSuccess; toff += kWaveK) {
-        e = cudaMemsetAsync(E->d_wcounter, 0, sizeof(int32_t), s);
-        if (e == cudaSuccess)
-            e = launch_wave_batch(E->d_winst, E->d_regions, E->d_region_inst, E->nregions,
-                                  E->d_wcounter, cur, toff, E->sms, s);
-        cur ^= 1;
+    for (int64_t k = 0; k < n && e == cudaSuccess; k += kWaveK) {
+        e = launch_tile_batch(E->tile, *cur, (int)k, (int)std::min<int64_t>(kWaveK, n - k), s);
+        *cur ^= 1;
     }
     if (e != cudaSuccess) return e;
     k_batch_advance_blocked<<<(std::max(1, E->cap_inst) + 255) / 256, 256, 0, s>>>(
-        E->d_inst, E->d_counts, kChunk);
+        E->d_inst, E->d_counts, (int)n);
     return cudaGetLastError();
 }
 
@@ -797,7 +791,8 @@ lbm_status build_batch_graph(lbm_engine *E) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(E->cap_main, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return fail_cuda(e, "batch: begin capture");
-    e = launch_blocked_chunk(E, E->cap_main);
+    int cur = E->wcur;
+    e = launch_blocked(E, kChunk, &cur, E->cap_main);
     if (one_step_instances(E) > 0)
         for (int s = 0; s < kChunk && e == cudaSuccess; ++s)
             e = launch_batch_step(E, E->cap_main, E->cap_side);
@@ -843,35 +838,17 @@ lbm_status engine_steps(lbm_engine *E, int64_t nsteps) {
                 if (e != cudaSuccess) return fail_cuda(e, "batch: launch");
             }
         E->launches += per_step * rest;
-        // the blocked instances take the rest of the steps with their own
-        // launches, as lbm_step would: blocked launches, then one-step ones
-        for (auto &I : E->inst) {
-            if (!I.blocked) continue;
-            lbm_solver *h = I.h;
-            for (int64_t k = 0; k < rest && e == cudaSuccess;) {
-                if (rest - k >= kWaveK) {
-                    e = launch_wave(h->L, h->S, h->wave, h->cur, (int)k, E->stream);
-                    k += kWaveK;
-                    E->launches += 1;
-                } else {
-                    e = launch_step(h->storage, h->L, h->S, h->cur, (int)k, E->stream, nullptr,
-                                    nullptr, nullptr, nullptr);
-                    k += 1;
-                    E->launches += kernels_per_step(h->L);
-                }
-                h->cur ^= 1;
-            }
-            if (e == cudaSuccess) e = launch_advance(h->S, rest, E->stream);
-            if (e != cudaSuccess) return fail_cuda(e, "batch: blocked instance launch");
-            E->launches += 1;
-            E->wcur = h->cur;  // the same for every blocked instance
+        if (E->nblocked > 0) {
+            e = launch_blocked(E, rest, &E->wcur, E->stream);
+            if (e != cudaSuccess) return fail_cuda(e, "batch: tile launch");
+            E->launches += (rest + kWaveK - 1) / kWaveK + 1;
         }
     }
     E->step_count += nsteps;
     for (auto &I : E->inst) {
         I.done = E->server ? std::min(I.steps, I.done + nsteps) : I.done + nsteps;
         I.h->time = I.done;
-        if (!I.blocked) I.h->cur = (int)(I.done & 1);
+        I.h->cur = I.blocked ? E->wcur : (int)(I.done & 1);
     }
     return LBM_OK;
 }
@@ -892,38 +869,24 @@ lbm_status engine_init(lbm_engine *E, int storage, void *stream) {
     return LBM_OK;
 }
 
-// The batched kernels step every instance one step per launch, so instances
-// are created without the tables of the temporally blocked kernel; each keeps
-// the streaming form its descriptor asks for.
+// The batched kernels step the instances themselves, so these are created
+// without a blocked form of their own; each keeps the streaming form its
+// descriptor asks for.
 lbm_desc one_step(const lbm_desc &d) {
     lbm_desc o = d;
     o.time_block = 1;
     return o;
 }
 
-// Rows of the strip segments a blocked batch instance is cut into: long
-// enough that the 3 kWaveK - 3 rows of a segment's pipeline fill and drain
-// stay a small part of it, short enough that a batch holds many more segments
-// than the device has SMs.
-constexpr int kBatchSegmentRows = 768;
-
-// Whether an instance of the lockstep batch takes the temporally blocked
-// kernel: FP32 storage, two population buffers and at least kWaveC columns.
+// Whether an instance of the lockstep batch is stepped in register tiles: FP32
+// storage, two population buffers and at least kWaveC columns.
 bool batch_blocked(const lbm_engine *E, const lbm_desc &d) {
     return !E->server && d.storage == LBM_F32 && d.streaming == LBM_STREAM_TWO_BUFFERS &&
-           d.nx >= kWaveC;
-}
-
-// The descriptor an instance is created from: the blocked form for the
-// instances batch_blocked() picks, one step per launch for the others.
-lbm_desc instance_desc(const lbm_engine *E, const lbm_desc &d_in) {
-    lbm_desc o = one_step(d_in);
-    if (batch_blocked(E, d_in)) o.time_block = LBM_TIME_BLOCK;
-    return o;
+           d.nx >= kWaveC && tile_supported();
 }
 
 // Admit one instance, from tables already validated and classified (d is the
-// instance's descriptor, instance_desc()), into the arena; LBM_ERR_NOMEM if it
+// instance's descriptor, one_step()), into the arena; LBM_ERR_NOMEM if it
 // does not fit now, and the tables are then left as they were.  Server
 // instances are created deferred: their uploads are queued behind the steps
 // already queued, with no wait on the host.
@@ -951,14 +914,7 @@ lbm_status admit_prepared(lbm_engine *E, const lbm_desc &d, Tables &t, const Uni
         return LBM_ERR_NOMEM;
     }
     lbm_handle h = nullptr;
-    int plan_blocks = 0;
-    if (d.time_block == LBM_TIME_BLOCK) {
-        const int strips = (d.nx + kWaveW - 1) / kWaveW;
-        const int segments = std::max(1, (d.ny + kBatchSegmentRows / 2) / kBatchSegmentRows);
-        plan_blocks = strips * segments;
-    }
     CreateOptions opt;
-    opt.plan_blocks = plan_blocks;
     opt.deferred = E->server;
     st = create_prepared(&d, std::move(t), u, E->stream, E->arena.base() + off, bytes, opt, &h);
     if (st != LBM_OK) {
@@ -967,8 +923,7 @@ lbm_status admit_prepared(lbm_engine *E, const lbm_desc &d, Tables &t, const Uni
     }
     Instance I;
     I.id = id;
-    I.blocked = h->block == kWaveK;
-    I.plan_blocks = plan_blocks;
+    I.blocked = batch_blocked(E, d);
     I.h = h;
     I.off = off;
     I.bytes = bytes;
@@ -981,7 +936,7 @@ lbm_status admit_prepared(lbm_engine *E, const lbm_desc &d, Tables &t, const Uni
 
 // Admit one instance from its descriptor (the lockstep batch).
 lbm_status admit(lbm_engine *E, const lbm_desc &d_in, int64_t id, int64_t steps) {
-    const lbm_desc d = instance_desc(E, d_in);
+    const lbm_desc d = one_step(d_in);
     Tables t;
     Units u;
     lbm_status st = prepare(&d, &t, &u);
@@ -1113,10 +1068,7 @@ lbm_engine::~lbm_engine() {
     requests.clear();  // waits for the workers of requests never admitted
     for (auto &g : graph)
         if (g) cudaGraphExecDestroy(g);
-    if (d_winst) cudaFree(d_winst);
-    if (d_regions) cudaFree(d_regions);
-    if (d_region_inst) cudaFree(d_region_inst);
-    if (d_wcounter) cudaFree(d_wcounter);
+    if (d_tile) cudaFree(d_tile);
     if (d_inst) cudaFree(d_inst);
     if (d_tiles) cudaFree(d_tiles);
     if (d_bmap) cudaFree(d_bmap);
@@ -1146,7 +1098,7 @@ extern "C" lbm_status lbm_batch_create(const lbm_desc *descs, int32_t count, voi
     uint64_t total = 0;
     for (int32_t i = 0; i < count; ++i) {
         uint64_t b = 0;
-        const lbm_desc di = instance_desc(E.get(), descs[i]);
+        const lbm_desc di = one_step(descs[i]);
         st = lbm_workspace_size(&di, &b);
         if (st != LBM_OK) return st;
         total += (b + 255) / 256 * 256;

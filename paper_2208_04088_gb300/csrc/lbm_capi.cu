@@ -230,7 +230,17 @@ extern "C" lbm_status lbm_workspace_size(const lbm_desc *desc, uint64_t *bytes) 
 
 extern "C" lbm_status lbm_create(const lbm_desc *desc, void *stream, void *workspace,
                                  uint64_t workspace_bytes, lbm_handle *out) {
-    return lbm::create_solver(desc, stream, workspace, workspace_bytes, 0, out);
+    set_error("");
+    if (!out) {
+        set_error("lbm_create: NULL output handle");
+        return LBM_ERR_ARG;
+    }
+    *out = nullptr;
+    Tables t;
+    Units u;
+    lbm_status st = prepare(desc, &t, &u);
+    if (st != LBM_OK) return st;
+    return create_prepared(desc, std::move(t), u, stream, workspace, workspace_bytes, CreateOptions(), out);
 }
 
 namespace lbm {
@@ -292,29 +302,11 @@ uint64_t workspace_bytes_for(const lbm_desc &d, const Tables &t, const Units &u)
     return layout(t, d.storage, u.lam != u.mu, block, d.streaming == LBM_STREAM_IN_PLACE).total;
 }
 
-lbm_status create_solver(const lbm_desc *desc, void *stream, void *workspace,
-                         uint64_t workspace_bytes, int plan_blocks, lbm_handle *out) {
-    set_error("");
-    if (!out) {
-        set_error("lbm_create: NULL output handle");
-        return LBM_ERR_ARG;
-    }
-    *out = nullptr;
-    Tables t;
-    Units u;
-    lbm_status st = prepare(desc, &t, &u);
-    if (st != LBM_OK) return st;
-    CreateOptions opt;
-    opt.plan_blocks = plan_blocks;
-    return create_prepared(desc, std::move(t), u, stream, workspace, workspace_bytes, opt, out);
-}
-
 lbm_status create_prepared(const lbm_desc *desc, Tables &&tab, const Units &units, void *stream,
                            void *workspace, uint64_t workspace_bytes, const CreateOptions &opt,
                            lbm_handle *out) {
     set_error("");
     *out = nullptr;
-    const int plan_blocks = opt.plan_blocks;
     lbm_solver *h = new lbm_solver();
     h->tab = std::move(tab);
     h->units = units;
@@ -412,7 +404,7 @@ lbm_status create_prepared(const lbm_desc *desc, Tables &&tab, const Units &unit
     // form: 8 steps of a 64^2 plate in 17 us against 35 us one step at a time,
     // of a 1024 x 512 plate 43 against 57, and with lambda != mu 4 steps of
     // the 2048^2 crack in 240 us against 364 (the strip kernel: 349).
-    if (e == cudaSuccess && opt.plan_blocks <= 0 && desc->time_block == 0 && h->block == 1 &&
+    if (e == cudaSuccess && desc->time_block == 0 && h->block == 1 &&
         h->storage == LBM_F32 && !in_place)
         e = tile_create(h);
     if (e == cudaSuccess && h->block > 1 && h->tile.shape < 0) {
@@ -424,9 +416,8 @@ lbm_status create_prepared(const lbm_desc *desc, Tables &&tab, const Units &unit
             }
             h->block = 1;  // default: fall back to one step per launch
         } else {
-            e = wave_prepare(h->tab, h->L, S, &h->wave, h->stream, plan_blocks);
-            if (e == cudaSuccess && plan_blocks <= 0)
-                e = wave_calibrate(h->tab, h->L, S, &h->wave, h->stream);
+            e = wave_prepare(h->tab, h->L, S, &h->wave, h->stream);
+            if (e == cudaSuccess) e = wave_calibrate(h->tab, h->L, S, &h->wave, h->stream);
             if (e == cudaSuccess) e = launch_reset(h->storage, h->L, S, h->stream);
         }
     }

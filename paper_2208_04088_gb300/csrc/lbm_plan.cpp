@@ -214,21 +214,6 @@ std::vector<int4> wave_plan(const Tables &t, int sms) {
     return cut_strips(br, nstrips, ny, std::max(sms, nstrips), cost);
 }
 
-std::vector<double> wave_plan_costs(const Tables &t, const std::vector<int4> &plan) {
-    const int nstrips = (t.nx + kPW - 1) / kPW;
-    const StripRows br = strip_rows(t, nstrips);
-    std::vector<double> out;
-    out.reserve(plan.size());
-    for (const int4 &b : plan) {
-        const int sx = b.x / kPW, a = b.y, e = b.y + b.z;
-        const auto &r = br.row[sx];
-        const size_t lo = std::lower_bound(r.begin(), r.end(), a - kPK) - r.begin();
-        const size_t hi = std::lower_bound(r.begin(), r.end(), e + kPK) - r.begin();
-        out.push_back((double)(e - a + 3 * kPK - 3) + kBlockCost + (br.pre[sx][hi] - br.pre[sx][lo]));
-    }
-    return out;
-}
-
 namespace {
 
 // Measured plans of this process, by lattice: a lattice created again (same
@@ -485,6 +470,8 @@ bool tile_plan(const Tables &t, bool wall_node, int shape, TilePlan *p) {
 
 namespace {
 
+}  // namespace
+
 // Modelled time (us) of one launch with a shape: every tile costs a fixed part
 // (copy in, store) and per step a part for its nodes, one for having boundary
 // rules at all (two more barriers and a link's dependent chain) and one per
@@ -534,8 +521,6 @@ double tile_time(const Tables &t, int shape, bool grad, int sms) {
     }
     return std::max(end, (total + (double)without * plain) / sms + 0.5 * plain);
 }
-
-}  // namespace
 
 void tile_choose(const Tables &t, bool grad, bool wall_node, int sms, TilePlan *p) {
     // One step per launch: bound by launches (two kernels beside each other,

@@ -448,6 +448,46 @@ __global__ void __launch_bounds__(kNT, 1)
                              sm);
 }
 
+// The tiles of many lattices in one launch (a batch, lambda = mu): a tile's
+// instance supplies its buffers, tables and lattice parameters.
+template <int LPR, int R>
+__global__ void __launch_bounds__(kNT, 1)
+    k_tile_batch(const TileInst *__restrict__ insts, const TileRec *__restrict__ tiles,
+                 const uint32_t *__restrict__ pubs, const TileLink *__restrict__ links, int cur,
+                 int toff, int nsteps) {
+    extern __shared__ __align__(1024) unsigned char sm[];
+    __shared__ __align__(16) Lattice s_L;
+    release_next();
+    const TileRec rec = tiles[blockIdx.x];
+    const TileInst *I = insts + rec.inst;
+    constexpr int kWords = (int)(sizeof(Lattice) / 4);
+    if (threadIdx.x < kWords)
+        reinterpret_cast<uint32_t *>(&s_L)[threadIdx.x] =
+            reinterpret_cast<const uint32_t *>(&I->L)[threadIdx.x];
+    __syncthreads();
+    tile_steps<LPR, R, false>(&I->map[cur], I->f[cur ^ 1], I->uc, I->cls, rec, pubs, links, I->bcs, s_L,
+                              I->time, toff, nsteps, I->status, sm);
+}
+
+template <int LPR, int R> cudaError_t batch_shape(const TileBatch &B, int cur, int toff, int nsteps,
+                                                  cudaStream_t s) {
+    static const cudaError_t attr_set = cudaFuncSetAttribute(
+        k_tile_batch<LPR, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Shape<LPR, R>::kSmem);
+    if (attr_set != cudaSuccess || B.ntiles <= 0) return attr_set;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)B.ntiles);
+    cfg.blockDim = dim3(kNT);
+    cfg.dynamicSmemBytes = Shape<LPR, R>::kSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_tile_batch<LPR, R>, B.insts, B.tiles, B.pubs, B.links, cur, toff,
+                              nsteps);
+}
+
 template <int LPR, int R, bool GRAD>
 cudaError_t launch_shape(const Lattice &L, const DevState &S, const TileDev &T, int cur, int toff,
                          int nsteps, cudaStream_t s) {
@@ -467,14 +507,20 @@ cudaError_t launch_shape(const Lattice &L, const DevState &S, const TileDev &T, 
                               S.status);
 }
 
-template <int LPR, int R> cudaError_t prepare_shape(const Lattice &L, const DevState &S, TileDev *T) {
+template <int LPR, int R>
+bool encode_shape(const Lattice &L, const DevState &S, CUtensorMap map[2]) {
     using Sh = Shape<LPR, R>;
     const cuuint64_t dims[3] = {(cuuint64_t)L.nx, (cuuint64_t)L.ny, 9};
     const cuuint64_t str[2] = {(cuuint64_t)L.pitch * 4, (cuuint64_t)L.fplane * 4};
     const cuuint32_t box[3] = {(cuuint32_t)Sh::W, (cuuint32_t)Sh::H, 9};
     for (int b = 0; b < 2; ++b)
-        if (!encode(&T->map[b], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, S.f[b], dims, str, box))
-            return cudaErrorInvalidValue;
+        if (!encode(&map[b], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, S.f[b], dims, str, box)) return false;
+    return true;
+}
+
+template <int LPR, int R> cudaError_t prepare_shape(const Lattice &L, const DevState &S, TileDev *T) {
+    using Sh = Shape<LPR, R>;
+    if (!encode_shape<LPR, R>(L, S, T->map)) return cudaErrorInvalidValue;
     return L.grad ? cudaFuncSetAttribute(k_tile<LPR, R, true>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::kSmem)
                   : cudaFuncSetAttribute(k_tile<LPR, R, false>,
@@ -508,6 +554,24 @@ cudaError_t launch_tile(const Lattice &L, const DevState &S, const TileDev &T, i
     }
 #undef LBM_TILE
     return cudaErrorInvalidValue;
+}
+
+bool tile_maps(const Lattice &L, const DevState &S, int shape, CUtensorMap map[2]) {
+    switch (shape) {
+        case 0: return encode_shape<16, 1>(L, S, map);
+        case 1: return encode_shape<32, 2>(L, S, map);
+        case 2: return encode_shape<32, 3>(L, S, map);
+        default: return encode_shape<32, 4>(L, S, map);
+    }
+}
+
+cudaError_t launch_tile_batch(const TileBatch &B, int cur, int toff, int nsteps, cudaStream_t s) {
+    switch (B.shape) {
+        case 0: return batch_shape<16, 1>(B, cur, toff, nsteps, s);
+        case 1: return batch_shape<32, 2>(B, cur, toff, nsteps, s);
+        case 2: return batch_shape<32, 3>(B, cur, toff, nsteps, s);
+        default: return batch_shape<32, 4>(B, cur, toff, nsteps, s);
+    }
 }
 
 }  // namespace lbm

@@ -433,35 +433,6 @@ __device__ __forceinline__ void wave_region(
         atomicOr(status, 2u);
         for (int j = last_waited + 1; j <= j_issued; ++j) wait_row(j, kDefaultWaitNs);
     }
-    // every copy has been waited for: the barriers are released, so that the
-    // block can initialise them again for its next region
-    if (tid == 0)
-        for (int q = 0; q < kNI; ++q) mbar_inval(bar0 + 8u * q);
-}
-
-// One launch over the regions of many lattices (a batch): a persistent grid
-// whose blocks take regions from an atomic counter; each region's instance
-// record supplies its tensor maps and buffers, and its lattice parameters are
-// staged in shared memory.
-__global__ void __launch_bounds__(kThreads, 1)
-    k_wave_batch(const WaveInst *__restrict__ insts, const int4 *__restrict__ regions,
-                 const int32_t *__restrict__ region_inst, int nregions,
-                 int32_t *__restrict__ counter, int cur, int toff) {
-    extern __shared__ __align__(1024) unsigned char sm[];
-    __shared__ int s_r;
-    __shared__ __align__(16) Lattice s_L;
-    for (;;) {
-        if (threadIdx.x == 0) s_r = atomicAdd(counter, 1);
-        __syncthreads();
-        const int r = s_r;
-        if (r >= nregions) break;
-        const WaveInst *I = insts + region_inst[r];
-        if (threadIdx.x == 0) s_L = I->L;
-        __syncthreads();
-        wave_region(&I->tf[cur], &I->tnw, &I->tu, I->f[cur ^ 1], I->uc, I->blinks, I->bcs, s_L,
-                    I->time, toff, regions[r], I->status, nullptr, sm);
-        __syncthreads();  // the next region reuses the shared memory
-    }
 }
 
 // One launch: kWaveK steps of every material node of one lattice; block b
@@ -931,7 +902,7 @@ bool wave_supported(const Lattice &L) {
 }
 
 cudaError_t wave_prepare(const Tables &t, const Lattice &L, const DevState &S, WaveMaps *m,
-                         cudaStream_t s, int plan_blocks) {
+                         cudaStream_t s) {
     const int64_t n = L.plane;
     k_nw_fill<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(S.cls, S.nw, n);
     if (L.nb > 0)
@@ -959,24 +930,12 @@ cudaError_t wave_prepare(const Tables &t, const Lattice &L, const DevState &S, W
                : cudaFuncSetAttribute(k_wave, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)kSmem);
     if (e != cudaSuccess) return e;
-    const std::vector<int4> plan = wave_plan(t, plan_blocks > 0 ? plan_blocks : device_sms());
+    const std::vector<int4> plan = wave_plan(t, device_sms());
     m->nblocks = (int)plan.size();
     if (plan.empty() || plan.size() > wave_table_entries(t.nx, t.ny)) return cudaErrorInvalidValue;
     // pageable source: the copy is staged before the call returns
     return cudaMemcpyAsync(S.wave_tab, plan.data(), plan.size() * sizeof(int4),
                            cudaMemcpyHostToDevice, s);
-}
-
-cudaError_t launch_wave_batch(const WaveInst *insts, const int4 *regions, const int32_t *region_inst,
-                              int nregions, int32_t *counter, int cur, int toff, int sms,
-                              cudaStream_t s) {
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_wave_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-    if (attr != cudaSuccess) return attr;
-    if (nregions <= 0) return cudaSuccess;
-    k_wave_batch<<<(unsigned)std::min(sms, nregions), kThreads, kSmem, s>>>(
-        insts, regions, region_inst, nregions, counter, cur, toff);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_wave(const Lattice &L, const DevState &S, const WaveMaps &m, int cur, int toff,
