@@ -157,12 +157,9 @@ typedef struct {
     int32_t wall_values; /* lbm_wall_values */
     int32_t time_block;  /* time steps fused into one kernel launch:
                             0  library default, the faster form: with FP32 storage
-                               and two buffers several steps per launch, by the
-                               strip kernel of LBM_TIME_BLOCK (lambda = mu, at least
-                               2^21 nodes, nx >= 128, at most one boundary node per
-                               800 nodes that is not on a box edge or crack face)
-                               or in register tiles (the other lattices, unless
-                               walls are everywhere); else 1
+                               and two buffers LBM_TIME_BLOCK steps per launch (4
+                               when lambda != mu) in register tiles, unless walls
+                               are everywhere in the lattice; else 1
                             1  one launch per step (bulk and boundary-list kernels)
                             LBM_TIME_BLOCK  temporal blocking: each launch carries
                                LBM_TIME_BLOCK steps (4 when lambda != mu, whose
@@ -218,8 +215,8 @@ lbm_status lbm_geom_build(const lbm_geom *geom, uint8_t *node_type, lbm_link *li
 /* Device bytes a handle for `desc` needs (distributions, displacement,
  * tables, field staging).  Host tables are validated as in lbm_create.  The
  * tables of the register tiles come on top: lbm_create allocates them itself
- * (about 100 bytes per boundary node and 32 per tile) and, if it cannot,
- * steps one step per launch. */
+ * (about 100 bytes per boundary node and 32 per tile) and, if it cannot, steps
+ * in strips (lambda = mu, large lattices) or one step per launch. */
 lbm_status lbm_workspace_size(const lbm_desc *desc, uint64_t *bytes);
 
 /* Create a solver: validates and classifies the tables on the host, copies

@@ -545,15 +545,18 @@ lbm_status build_tile_tables(lbm_engine *E) {
                      [](const TileRec &a, const TileRec &b) { return a.nlink > b.nlink; });
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t bi = up(sizeof(TileInst) * inst.size()), bt = up(sizeof(TileRec) * all.tiles.size());
-    const size_t bp = up(sizeof(uint32_t) * all.pubs.size()), bl = sizeof(TileLink) * all.links.size();
-    cudaError_t e = cudaMalloc(&E->d_tile, bi + bt + bp + bl);
+    const size_t bp = up(sizeof(uint32_t) * all.pubs.size()), bl = up(sizeof(TileLink) * all.links.size());
+    cudaError_t e = cudaMalloc(&E->d_tile, bi + bt + bp + bl + 256);
     if (e != cudaSuccess) return fail_cuda(e, "batch: tile tables");
     char *m = static_cast<char *>(E->d_tile);
     E->tile.shape = all.shape;
+    E->tile.sms = E->sms;
+    for (const TileInst &w : inst) E->tile.force |= w.L.fx != 0.0f || w.L.fy != 0.0f;
     E->tile.insts = reinterpret_cast<const TileInst *>(m);
     E->tile.tiles = reinterpret_cast<const TileRec *>(m + bi);
     E->tile.pubs = reinterpret_cast<const uint32_t *>(m + bi + bt);
     E->tile.links = reinterpret_cast<const TileLink *>(m + bi + bt + bp);
+    E->tile.counter = reinterpret_cast<int32_t *>(m + bi + bt + bp + bl);
     // sets the kernel's shared-memory limit (outside any capture); launches nothing
     e = launch_tile_batch(E->tile, 0, 0, 0, E->stream);
     E->tile.ntiles = (int)all.tiles.size();
@@ -568,7 +571,9 @@ lbm_status build_tile_tables(lbm_engine *E) {
         e = cudaMemcpyAsync(m + bi + bt, all.pubs.data(), sizeof(uint32_t) * all.pubs.size(),
                             cudaMemcpyHostToDevice, E->stream);
     if (e == cudaSuccess && !all.links.empty())
-        e = cudaMemcpyAsync(m + bi + bt + bp, all.links.data(), bl, cudaMemcpyHostToDevice, E->stream);
+        e = cudaMemcpyAsync(m + bi + bt + bp, all.links.data(), sizeof(TileLink) * all.links.size(),
+                            cudaMemcpyHostToDevice, E->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(E->tile.counter, 0, 256, E->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(E->stream);  // the host vectors die here
     if (e != cudaSuccess) return fail_cuda(e, "batch: tile tables upload");
     return LBM_OK;

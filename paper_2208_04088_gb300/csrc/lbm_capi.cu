@@ -49,13 +49,12 @@ int steps_per_launch(const lbm_desc &d, const Tables &t, const Units &u) {
     const int k = u.lam == u.mu ? kWaveK : kWaveGradK;
     if (d.time_block == 1) return 1;
     if (d.time_block == LBM_TIME_BLOCK) return ok ? k : 0;
-    // The library default: blocked where that measured faster on GB300 --
-    // lambda = mu (with lambda != mu the blocked kernel carries 4 levels and
-    // its collision warps set each row's time: 48 vs 47 GLUPS on the 2048^2
-    // crack, too small a margin to make it the default), lattices of at
+    // What the default's workspace is laid out for, and what it steps with
+    // should the tables of its register tiles not be had: strips where they
+    // measured faster than one step per launch -- lambda = mu, lattices of at
     // least 2^21 nodes (below, the fill of each block's row pipeline dominates:
     // 1024^2 plate 57 vs 80 GLUPS), and at most one boundary node off box edges
-    // and crack faces per 800 nodes: the blocked kernel updates those eight
+    // and crack faces per 800 nodes: the strip kernel updates those eight
     // lanes to a node at every level (2048^2 plates with a hole: radius 512,
     // one per 1022 nodes, 74 vs 59 GLUPS; radius 900, one per 582, 34 vs 48).
     const int64_t nodes = (int64_t)t.nx * t.ny;
@@ -111,6 +110,7 @@ Lattice make_lattice(const Tables &t, const Units &u, int storage) {
     L.fplane = L.plane;
     L.omega = (float)(1.0 / u.tau);
     L.src = (float)(1.0 - 1.0 / (2.0 * u.tau));
+    L.src_tau = (float)((u.tau - 0.5) / 3.0);
     L.fx = (float)u.fx;
     L.fy = (float)u.fy;
     L.mu_m_lam = (float)(u.mu - u.lam);
@@ -271,7 +271,7 @@ static cudaError_t tile_create(lbm_solver *h) {
     const size_t bp = align256(plan.pubs.size() * sizeof(uint32_t));
     const size_t bl = align256(plan.links.size() * sizeof(TileLink));
     TileDev &T = h->tile;
-    if (cudaMalloc(&T.mem, bt + bp + bl) != cudaSuccess) {
+    if (cudaMalloc(&T.mem, bt + bp + bl + 256) != cudaSuccess) {
         cudaGetLastError();
         T.mem = nullptr;
         return cudaSuccess;
@@ -280,8 +280,10 @@ static cudaError_t tile_create(lbm_solver *h) {
     T.tiles = reinterpret_cast<const TileRec *>(m);
     T.pubs = reinterpret_cast<const uint32_t *>(m + bt);
     T.links = reinterpret_cast<const TileLink *>(m + bt + bp);
+    T.counter = reinterpret_cast<int32_t *>(m + bt + bp + bl);
     T.ntiles = (int)plan.tiles.size();
     T.shape = plan.shape;
+    T.sms = device_sms();
     // pageable sources: the copies are staged before the calls return
     cudaError_t e = cudaMemcpyAsync(m, plan.tiles.data(), plan.tiles.size() * sizeof(TileRec),
                                     cudaMemcpyHostToDevice, h->stream);
@@ -291,6 +293,7 @@ static cudaError_t tile_create(lbm_solver *h) {
     if (e == cudaSuccess && !plan.links.empty())
         e = cudaMemcpyAsync(m + bt + bp, plan.links.data(), plan.links.size() * sizeof(TileLink),
                             cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(T.counter, 0, 256, h->stream);
     if (e == cudaSuccess) e = tile_prepare(h->L, h->S, &T);
     h->block = h->L.grad ? kWaveGradK : kWaveK;
     return e;
@@ -400,11 +403,12 @@ lbm_status create_prepared(const lbm_desc *desc, Tables &&tab, const Units &unit
         e = cudaMemcpyAsync(S.bcs, t.bcs.data(), t.bcs.size() * sizeof(BCDev),
                             cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = launch_reset(h->storage, h->L, S, h->stream);
-    // The default takes register tiles wherever the strip kernel is not its
-    // form: 8 steps of a 64^2 plate in 17 us against 35 us one step at a time,
-    // of a 1024 x 512 plate 43 against 57, and with lambda != mu 4 steps of
-    // the 2048^2 crack in 240 us against 364 (the strip kernel: 349).
-    if (e == cudaSuccess && desc->time_block == 0 && h->block == 1 &&
+    // The default takes register tiles wherever their modelled time is below
+    // one step per launch: 8 steps of a 64^2 plate in 17 us against 35, of a
+    // 1024 x 512 plate in 34 against 57, of the 2048^2 crack in 192 us against
+    // 300 in strips (k_wave, 538 one step at a time), and with lambda != mu 4
+    // steps of the crack in 198 us against 364 (strips: 349).
+    if (e == cudaSuccess && desc->time_block == 0 &&
         h->storage == LBM_F32 && !in_place)
         e = tile_create(h);
     if (e == cudaSuccess && h->block > 1 && h->tile.shape < 0) {

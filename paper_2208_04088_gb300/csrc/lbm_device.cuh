@@ -164,16 +164,43 @@ template <> __device__ __forceinline__ float splat<float>(float c) { return c; }
 template <> __device__ __forceinline__ F2 splat<F2>(float c) { return f2(c, c); }
 
 // ---------------------------------------------------------------------------
+// The arithmetic of a storage form.  The two evaluate the same collision with
+// different rounding orders: kSums32 needs 39 operations per node without a
+// source, kSums16 65.  16-bit storage keeps the longer one: a stored value that
+// rounds the other way would move its results by their own error (1e-3).
+enum : int { kSums16 = 0, kSums32 = 1 };
+template <class T> constexpr int kSumsOf = std::is_same<T, float>::value ? kSums32 : kSums16;
+
 // Raw moments m_pq = sum_i f_i c_ix^p c_iy^q (p, q in 0..2) of the nine
 // populations.  D2Q9 is the tensor product of {-1, 0, 1} in x and y, so the
 // transform is two passes of the 1-D map (a-, a0, a+) -> (a- + a0 + a+,
-// a+ - a-, a+ + a-), whose inverse has only the coefficients 1 and 1/2: the
-// round trip adds nothing but additions to the rounding.
+// a+ - a-, a+ + a-): it adds nothing but additions to the rounding.
 template <class V> struct RawT {
     V m00, m10, m01, m20, m02, m11, m21, m12, m22;
 };
 using Raw = RawT<float>;
 
+// kSums32: every sum of three takes the sum of its outer two, so a 1-D map is
+// three operations.
+template <class V> __device__ __forceinline__ RawT<V> raw_sums(const V f[9]) {
+    // rows c_y = -1: (f7, f4, f8); c_y = 0: (f3, f0, f1); c_y = +1: (f6, f2, f5)
+    const V a2 = radd(f[8], f[7]), a1 = rsub(f[8], f[7]), a0 = radd(a2, f[4]);
+    const V b2 = radd(f[1], f[3]), b1 = rsub(f[1], f[3]), b0 = radd(b2, f[0]);
+    const V c2 = radd(f[5], f[6]), c1 = rsub(f[5], f[6]), c0 = radd(c2, f[2]);
+    RawT<V> m;
+    m.m02 = radd(c0, a0);
+    m.m00 = radd(m.m02, b0);
+    m.m01 = rsub(c0, a0);
+    m.m12 = radd(c1, a1);
+    m.m10 = radd(m.m12, b1);
+    m.m11 = rsub(c1, a1);
+    m.m22 = radd(c2, a2);
+    m.m20 = radd(m.m22, b2);
+    m.m21 = rsub(c2, a2);
+    return m;
+}
+
+// kSums16.
 template <class V> __device__ __forceinline__ RawT<V> raw_moments(const V f[9]) {
     // rows c_y = -1: (f7, f4, f8); c_y = 0: (f3, f0, f1); c_y = +1: (f6, f2, f5)
     const V a0 = radd(radd(f[7], f[4]), f[8]), a1 = rsub(f[8], f[7]), a2 = radd(f[8], f[7]);
@@ -219,8 +246,12 @@ struct Mom {
     float dr, mx, my, pxx, pyy, pxy;
 };
 
-__device__ __forceinline__ Mom moments(const float f[9]) {
-    const Raw r = raw_moments(f);
+template <int kSums> __device__ __forceinline__ Mom moments(const float f[9]) {
+    Raw r;
+    if constexpr (kSums == kSums32)
+        r = raw_sums(f);
+    else
+        r = raw_moments(f);
     return Mom{r.m00, r.m10, r.m01, r.m20, r.m02, r.m11};
 }
 
@@ -262,26 +293,79 @@ __device__ __forceinline__ void collide_v(V f[9], V sx, V sy, V w, V s3, V &dr_o
     populations(m, f);
 }
 
+// kSums32: the collision changes only the moments m_xxy, m_xyy and m_xxyy (and j
+// by the source), so it is f plus the inverse transforms of those three
+// changes, formed from their negatives n = m - m^eq: corners take -omega/4 of
+// n_xxyy +- n_xxy +- n_xyy, the axis directions +omega/2 of n_xxyy +- their odd
+// one, the rest population -omega n_xxyy.  The factors are exact multiples of
+// one rounded omega, so rho, j and P lose nothing to them.  kSource: S enters
+// j, the odd moments with (1 - 1/(2 tau))/3 and the axis directions with S/2;
+// without it the operations whose result S = 0 leaves unchanged are left out.
+template <class V> struct Relax {
+    V w, w2, mw4, msrc;  // -omega, omega/2, -omega/4, -(tau - 1/2)/3
+};
+template <class V> __device__ __forceinline__ Relax<V> relax_of(const Lattice &L) {
+    return Relax<V>{splat<V>(-L.omega), splat<V>(rmul(0.5f, L.omega)), splat<V>(rmul(-0.25f, L.omega)),
+                    splat<V>(-L.src_tau)};
+}
+
+template <bool kSource, class V>
+__device__ __forceinline__ void collide_sums(V f[9], V sx, V sy, const Relax<V> &c, V &dr_out, V &jx_out,
+                                             V &jy_out) {
+    const V mthird = splat<V>(-1.0f / 3.0f);
+    const RawT<V> m = raw_sums(f);
+    V jx = m.m10, jy = m.m01;
+    if constexpr (kSource) {
+        const V half = splat<V>(0.5f), mhalf = splat<V>(-0.5f);
+        jx = rfma(half, sx, jx);
+        jy = rfma(half, sy, jy);
+        f[1] = rfma(half, sx, f[1]);
+        f[3] = rfma(mhalf, sx, f[3]);
+        f[2] = rfma(half, sy, f[2]);
+        f[4] = rfma(mhalf, sy, f[4]);
+    }
+    V n21 = rfma(jy, mthird, m.m21), n12 = rfma(jx, mthird, m.m12);
+    if constexpr (kSource) {
+        n21 = rfma(c.msrc, sy, n21);
+        n12 = rfma(c.msrc, sx, n12);
+    }
+    const V n22 = rfma(rfma(m.m00, mthird, radd(m.m20, m.m02)), mthird, m.m22);
+    const V p = radd(n22, n21), q = rsub(n22, n21);
+    f[5] = rfma(c.mw4, radd(p, n12), f[5]);
+    f[6] = rfma(c.mw4, rsub(p, n12), f[6]);
+    f[7] = rfma(c.mw4, rsub(q, n12), f[7]);
+    f[8] = rfma(c.mw4, radd(q, n12), f[8]);
+    f[1] = rfma(c.w2, radd(n22, n12), f[1]);
+    f[3] = rfma(c.w2, rsub(n22, n12), f[3]);
+    f[2] = rfma(c.w2, p, f[2]);
+    f[4] = rfma(c.w2, q, f[4]);
+    f[0] = rfma(c.w, n22, f[0]);
+    dr_out = m.m00;
+    jx_out = jx;
+    jy_out = jy;
+}
+
+template <int kSums>
 __device__ __forceinline__ void collide(float f[9], float sx, float sy, const Lattice &L,
                                         float &dr_out, float &jx_out, float &jy_out) {
-    collide_v<float>(f, sx, sy, L.omega, rmul(L.src, 1.0f / 3.0f), dr_out, jx_out, jy_out);
+    if constexpr (kSums == kSums32)
+        collide_sums<true>(f, sx, sy, relax_of<float>(L), dr_out, jx_out, jy_out);
+    else
+        collide_v<float>(f, sx, sy, L.omega, rmul(L.src, 1.0f / 3.0f), dr_out, jx_out, jy_out);
 }
 
 // u(t+1) = u(t) + j/rho with Kahan compensation per component; w holds
 // (u_x, u_y, compensation_x, compensation_y).
 __device__ __forceinline__ void integrate_u_value(float4 &w, float jx, float jy, float rho) {
     // v = j/rho as j times one approximate reciprocal (relative error about
-    // 1e-7, far below the FP32 parity bound; no divisions)
-    const float ir = __fdividef(1.0f, rho);
-    const float vx = rmul(jx, ir), vy = rmul(jy, ir);
-    float y = rsub(vx, w.z);
-    float t = radd(w.x, y);
-    w.z = rsub(rsub(t, w.x), y);
-    w.x = t;
-    y = rsub(vy, w.w);
-    t = radd(w.y, y);
-    w.w = rsub(rsub(t, w.y), y);
-    w.y = t;
+    // 1e-7, far below the FP32 parity bound; no divisions); the two components
+    // in pairs (bit by bit the scalar operations)
+    float ir;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ir) : "f"(rho));
+    const F2 v = f2(rmul(jx, ir), rmul(jy, ir)), u = f2(w.x, w.y);
+    const F2 y = rsub(v, f2(w.z, w.w)), t = radd(u, y);
+    f2_split(rsub(rsub(t, u), y), w.z, w.w);
+    f2_split(t, w.x, w.y);
 }
 
 // 16-bit storage: u(t+1) = u(t) + j/rho without compensation; w holds
@@ -659,7 +743,7 @@ __device__ __forceinline__ void pull_boundary(const T *src, const BNode &b,
         const int64_t ku = up ? k - (int64_t)c_cy(i) * L.pitch - c_cx(i) : k;
         gy1[i] = Store<T>::ld(src + col_at<LAY>(ku, i, L), L.inv_scale);
     }
-    const Mom mx = moments(gx);
+    const Mom mx = moments<kSumsOf<T>>(gx);
     f[0] = gx[0];
 #pragma unroll
     for (int kk = 1; kk < 9; ++kk) {
@@ -679,7 +763,7 @@ __device__ __forceinline__ void pull_boundary(const T *src, const BNode &b,
             float gy[9];
 #pragma unroll
             for (int m = 0; m < 9; ++m) gy[m] = Store<T>::ld(src + col_at<LAY>(ku, m, L), L.inv_scale);
-            const Mom my = moments(gy);
+            const Mom my = moments<kSumsOf<T>>(gy);
             my_dr = my.dr;
             my_xx = my.pxx;
             my_yy = my.pyy;
@@ -696,7 +780,7 @@ __device__ __forceinline__ void pull_boundary(const T *src, const BNode &b,
 // pull_boundary.  `ld(m, dx, dy)` returns f_m^col(t-1) at the node offset by
 // (dx, dy); `link(i)` the link record of cut direction i; the masks are those
 // of BNode.  g0 receives f_0^col(x), which is f_0(x, t).
-template <class Ld, class Lk>
+template <int kSums, class Ld, class Lk>
 __device__ __forceinline__ float boundary8_pull(const Ld &ld, uint32_t cutm, uint32_t dirm,
                                                 uint32_t corm, uint32_t missm, int k,
                                                 const Lk &link, const BCDev *__restrict__ bcs,
@@ -722,14 +806,14 @@ __device__ __forceinline__ float boundary8_pull(const Ld &ld, uint32_t cutm, uin
         float gy[9];
 #pragma unroll
         for (int m = 0; m < 9; ++m) gy[m] = ld(m, cxk, cyk);
-        const Mom my = moments(gy);
+        const Mom my = moments<kSums>(gy);
         my_dr = my.dr;
         my_xx = my.pxx;
         my_yy = my.pyy;
         my_xy = my.pxy;
     }
     if (!cut) return pulled;
-    const Mom mx = moments(g);  // rho and P are collision invariants: those of f^col(x, t-1)
+    const Mom mx = moments<kSums>(g);  // rho and P are collision invariants: those of f^col(x, t-1)
     return cut_link_value(k, miss, (dirm & bit) != 0, (corm & bit) != 0, neu_ex, link(i), gk, gi,
                           gy_i, mx.dr, mx.pxx, mx.pyy, mx.pxy, my_dr, my_xx, my_yy, my_xy, bcs, tb,
                           L);
@@ -748,7 +832,7 @@ __device__ __forceinline__ float pull_boundary8(const T *src, const BNode &b, in
         return Store<T>::ld(src + col_at<LAY>(kn + (int64_t)dy * pitch + dx, m, L), inv);
     };
     auto link = [&](int i) { return links[i - 1]; };
-    return boundary8_pull(ld, b.cut, b.dirich, b.corner, b.miss, k, link, bcs, tb, L, f0);
+    return boundary8_pull<kSumsOf<T>>(ld, b.cut, b.dirich, b.corner, b.miss, k, link, bcs, tb, L, f0);
 }
 
 // Collision of a boundary node held one population per lane (group of eight
@@ -756,6 +840,7 @@ __device__ __forceinline__ float pull_boundary8(const T *src, const BNode &b, in
 // gathered on every lane and collide() runs on them.  Returns the
 // post-collision population of the lane's direction; on every lane f0_out,
 // jx, jy and dr are the node's rest population, momentum and density deviation.
+template <int kSums>
 __device__ __forceinline__ float boundary8_collide(float fk, float g0, int kdir, float sx,
                                                    float sy, const Lattice &L, float &f0_out,
                                                    float &jx, float &jy, float &dr) {
@@ -764,7 +849,7 @@ __device__ __forceinline__ float boundary8_collide(float fk, float g0, int kdir,
     f[0] = g0;
 #pragma unroll
     for (int m = 1; m < 9; ++m) f[m] = __shfl_sync(0xffffffffu, fk, base + m - 1);
-    collide(f, sx, sy, L, dr, jx, jy);
+    collide<kSums>(f, sx, sy, L, dr, jx, jy);
     float mine = f[1];
 #pragma unroll
     for (int q = 2; q < 9; ++q)
@@ -773,13 +858,13 @@ __device__ __forceinline__ float boundary8_collide(float fk, float g0, int kdir,
     return mine;
 }
 
-// Density deviation rho - rho0 of nine populations, summed as raw_moments
-// forms m00 (so it equals moments(f).dr bit for bit); one node or two.
+// Density deviation rho - rho0 of nine populations, summed as raw_sums forms
+// m00 (so it equals moments<kSums32>(f).dr bit for bit); one node or two.
 template <class V> __device__ __forceinline__ V density_of(const V f[9]) {
-    const V a0 = radd(radd(f[7], f[4]), f[8]);
-    const V b0 = radd(radd(f[3], f[0]), f[1]);
-    const V c0 = radd(radd(f[6], f[2]), f[5]);
-    return radd(radd(a0, b0), c0);
+    const V a0 = radd(radd(f[8], f[7]), f[4]);
+    const V b0 = radd(radd(f[1], f[3]), f[0]);
+    const V c0 = radd(radd(f[5], f[6]), f[2]);
+    return radd(radd(c0, a0), b0);
 }
 
 // The source coefficient (mu - lambda)/rho = (mu - lambda) times an
@@ -860,7 +945,7 @@ __device__ __forceinline__ float node_drho(const T *__restrict__ src,
     if (__ldg(cls + k) != kInterior) return rho[k];
     float f[9];
     pull_interior(src, k, L.pitch, L.fplane, L.inv_scale, f);
-    return moments(f).dr;
+    return moments<kSumsOf<T>>(f).dr;
 }
 
 // The nine incoming populations of a boundary node held one per lane (group
@@ -917,7 +1002,7 @@ __device__ __forceinline__ void interior_node(const T *src, T *dst, URec<T> *__r
     float sx = L.fx, sy = L.fy;
     if (L.grad) source_interior(rho, k, L.pitch, rho[k], L, sx, sy);
     float dr, jx, jy;
-    collide(f, sx, sy, L, dr, jx, jy);
+    collide<kSumsOf<T>>(f, sx, sy, L, dr, jx, jy);
 #pragma unroll
     for (int i = 0; i < 9; ++i) Store<T>::st(dst + out_at<LAY>(k, i, L), f[i], L.scale);
     if constexpr (std::is_same<T, __half>::value) {
@@ -959,7 +1044,7 @@ __device__ __forceinline__ void boundary8_node(const T *src, T *dst, URec<T> *__
     float sx = L.fx, sy = L.fy;
     if (L.grad) source_boundary8(src, cls, rho, b, kn, L, j, sx, sy);
     float fr, jx, jy, m00;
-    const float mine = boundary8_collide(fk, f0, kdir, sx, sy, L, fr, jx, jy, m00);
+    const float mine = boundary8_collide<kSumsOf<T>>(fk, f0, kdir, sx, sy, L, fr, jx, jy, m00);
     if (!live) return;
     if (stage) {
         stage[(int64_t)g * 9 + kdir] = mine;
@@ -987,7 +1072,7 @@ __device__ __forceinline__ void boundary8_node(const T *src, T *dst, URec<T> *__
 // population is read across a cut link (ld may only address the lattice);
 // without it those reads are issued unconditionally and their values replaced
 // (ld addresses rows with halo columns).
-template <bool kGuard, class Ld>
+template <bool kGuard, int kSums, class Ld>
 __device__ __forceinline__ void simple_pull(const Ld &ld, uint32_t cut, uint32_t dirich,
                                             uint32_t miss, const BLink &sl,
                                             const BCDev *__restrict__ bcs, float tb,
@@ -999,7 +1084,7 @@ __device__ __forceinline__ void simple_pull(const Ld &ld, uint32_t cut, uint32_t
 #pragma unroll
     for (int k = 1; k < 9; ++k)  // intact links (the cut ones are replaced below)
         f[k] = kGuard && ((cut >> opp(k)) & 1u) ? 0.0f : ld(k, -c_cx(k), -c_cy(k));
-    const Mom mx = moments(g);
+    const Mom mx = moments<kSums>(g);
     float kap, fac;
     link_kappa(0.5f, kap, fac);
     if (dirich) {
@@ -1036,7 +1121,7 @@ __device__ __forceinline__ void simple_pull(const Ld &ld, uint32_t cut, uint32_t
             float gy[9];
 #pragma unroll
             for (int m = 0; m < 9; ++m) gy[m] = ld(m, cxk, cyk);
-            const Mom my = moments(gy);
+            const Mom my = moments<kSums>(gy);
             const WallState st = wall_state(true, 0.5f, mx.dr, mx.pxx, mx.pyy, mx.pxy, my.dr,
                                             my.pxx, my.pyy, my.pxy, L);
             float ax, ay, axy;
@@ -1072,11 +1157,11 @@ __device__ __forceinline__ void simple_node(const T *src, T *dst, URec<T> *__res
     const int d0 = __ffs((int)(cut >> 1));  // first cut direction, 1..8
     const BLink sl = blinks[(int64_t)g * 8 + (d0 > 0 ? d0 - 1 : 0)];
     float f[9];
-    simple_pull<true>(GlobalRows<T>{src, k, L.pitch, L.fplane, L.inv_scale}, cut, b.dirich,
+    simple_pull<true, kSumsOf<T>>(GlobalRows<T>{src, k, L.pitch, L.fplane, L.inv_scale}, cut, b.dirich,
                       b.miss, sl, bcs, tb, L, f);
     URec<T> w = uc[k];
     float dr, jx, jy;
-    collide(f, L.fx, L.fy, L, dr, jx, jy);
+    collide<kSumsOf<T>>(f, L.fx, L.fy, L, dr, jx, jy);
 #pragma unroll
     for (int i = 0; i < 9; ++i) Store<T>::st(dst + i * L.fplane + k, f[i], L.scale);
     if constexpr (std::is_same<T, __half>::value) {

@@ -81,6 +81,7 @@ struct Lattice {
     float out_u, out_v, out_s;  // lattice -> physical units for the fields
     int32_t grad;               // lambda != mu: the source needs grad rho
     int32_t wall_node;          // Neumann wall values at the boundary node (no extrapolation)
+    float src_tau;              // tau src/3 = (tau - 1/2)/3
     int64_t fplane;             // elements per population plane: plane, or with
                                 // in-place streaming pitch * (ny + 2) (a ring of one node)
     int32_t in_place;           // one population buffer, AA pattern (lbm_desc.streaming)
@@ -302,10 +303,11 @@ void tile_choose(const Tables &t, bool grad, bool wall_node, int sms, TilePlan *
 // Device side of a plan (tables owned by the handle, outside its workspace).
 struct TileDev {
     CUtensorMap map[2];  // the population buffers, box of one tile
-    int shape = -1, ntiles = 0;
+    int shape = -1, ntiles = 0, sms = 1;
     const TileRec *tiles = nullptr;
     const uint32_t *pubs = nullptr;
     const TileLink *links = nullptr;
+    int32_t *counter = nullptr;  // tiles taken, blocks done (both 0 between launches)
     void *mem = nullptr;
 };
 // Device record of one instance of a batch stepped in tiles, and the tables of
@@ -321,11 +323,13 @@ struct TileInst {
     Lattice L;
 };
 struct TileBatch {
-    int shape = -1, ntiles = 0;
+    int shape = -1, ntiles = 0, sms = 1;
+    bool force = false;  // some instance has a body force
     const TileInst *insts = nullptr;
     const TileRec *tiles = nullptr;
     const uint32_t *pubs = nullptr;
     const TileLink *links = nullptr;
+    int32_t *counter = nullptr;  // as in TileDev
 };
 // The modelled time (us) of a launch with a shape on `sms` SMs.
 double tile_time(const Tables &t, int shape, bool grad, int sms);

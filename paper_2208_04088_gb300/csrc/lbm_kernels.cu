@@ -98,10 +98,10 @@ __global__ void __launch_bounds__(kBX *kBY, kPairMinBlocks<T>) k_interior_pair(c
 // own pulled populations, ring nodes by pulling theirs, boundary nodes from the
 // boundary density pass), then the central differences of grad rho feed the
 // source of Eq. (sourceterm).  No full-lattice density pass is needed.
-constexpr int kGY = 8;  // rows of the lambda != mu tile (16 measured slower)
+constexpr int kGX = 32, kGY = 8;  // the lambda != mu tile (16 rows measured slower)
 
 template <class T>
-__global__ void __launch_bounds__(kBX *kGY) k_interior_grad(const T *__restrict__ src,
+__global__ void __launch_bounds__(kGX *kGY) k_interior_grad(const T *__restrict__ src,
                                                             T *__restrict__ dst,
                                                             URec<T> *__restrict__ uc,
                                                             const uint8_t *__restrict__ cls,
@@ -110,29 +110,29 @@ __global__ void __launch_bounds__(kBX *kGY) k_interior_grad(const T *__restrict_
                                                             uint32_t *__restrict__ status,
                                                             const int64_t *__restrict__ time,
                                                             int toff) {
-    __shared__ float rs[kGY + 2][kBX + 2];
+    __shared__ float rs[kGY + 2][kGX + 2];
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const int x0 = blockIdx.x * kBX, y0 = blockIdx.y * kGY;
+    const int x0 = blockIdx.x * kGX, y0 = blockIdx.y * kGY;
     scales_of_step<T>(L, time, toff, x0 + tx == 0 && y0 + ty == 0);
     const int x = x0 + tx, y = y0 + ty;
-    // the ring: top and bottom rows (kBX + 2 each), left and right columns (kGY each)
-    const int tid = ty * kBX + tx;
-    constexpr int kRing = 2 * (kBX + 2) + 2 * kGY;
+    // the ring: top and bottom rows (kGX + 2 each), left and right columns (kGY each)
+    const int tid = ty * kGX + tx;
+    constexpr int kRing = 2 * (kGX + 2) + 2 * kGY;
     int hx = 0, hy = 0;
     int64_t kk = -1;  // lattice index of this thread's ring node, if any
     if (tid < kRing) {
-        if (tid < kBX + 2) {
+        if (tid < kGX + 2) {
             hx = tid;
             hy = 0;
-        } else if (tid < 2 * (kBX + 2)) {
-            hx = tid - (kBX + 2);
+        } else if (tid < 2 * (kGX + 2)) {
+            hx = tid - (kGX + 2);
             hy = kGY + 1;
-        } else if (tid < 2 * (kBX + 2) + kGY) {
+        } else if (tid < 2 * (kGX + 2) + kGY) {
             hx = 0;
-            hy = tid - 2 * (kBX + 2) + 1;
+            hy = tid - 2 * (kGX + 2) + 1;
         } else {
-            hx = kBX + 1;
-            hy = tid - 2 * (kBX + 2) - kGY + 1;
+            hx = kGX + 1;
+            hy = tid - 2 * (kGX + 2) - kGY + 1;
         }
         const int gx = x0 - 1 + hx, gy = y0 - 1 + hy;
         if (gx >= 0 && gx < L.nx && gy >= 0 && gy < L.ny) kk = (int64_t)gy * L.pitch + gx;
@@ -159,9 +159,9 @@ __global__ void __launch_bounds__(kBX *kGY) k_interior_grad(const T *__restrict_
         ring_int = true;
         pull_interior(src, kk, L.pitch, L.fplane, L.inv_scale, g);
     }
-    if (live) own = moments(f).dr;
+    if (live) own = moments<kSumsOf<T>>(f).dr;
     else if (c == kBoundary) own = rho[k];
-    if (ring_int) v = moments(g).dr;
+    if (ring_int) v = moments<kSumsOf<T>>(g).dr;
     else if (cr == kBoundary) v = rho[kk];
     rs[ty + 1][tx + 1] = own;
     if (tid < kRing) rs[hy][hx] = v;
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kBX *kGY) k_interior_grad(const T *__restrict_
     grad_source(own, rs[ty + 1][tx + 2], rs[ty + 1][tx], rs[ty + 2][tx + 1], rs[ty][tx + 1], true,
                 true, true, true, L, sx, sy);
     float dr, jx, jy;
-    collide(f, sx, sy, L, dr, jx, jy);
+    collide<kSumsOf<T>>(f, sx, sy, L, dr, jx, jy);
 #pragma unroll
     for (int i = 0; i < 9; ++i) Store<T>::st(dst + i * L.fplane + k, f[i], L.scale);
     if constexpr (std::is_same<T, __half>::value) {
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kBX *kBY) k_density_interior(const T *__restri
     if (cls[k] != kInterior) return;
     float f[9];
     pull_interior(src, k, L.pitch, L.fplane, L.inv_scale, f);
-    rho[k] = moments(f).dr;
+    rho[k] = moments<kSumsOf<T>>(f).dr;
 }
 
 template <class T>
@@ -267,15 +267,15 @@ __global__ void __launch_bounds__(kBB) k_density_boundary(const T *__restrict__ 
     const float tb = (float)(*time + toff - 1);
     float f[9];
     pull_boundary(src, b, blinks + (int64_t)m * 8, bcs, tb, L, f);
-    rho[(int64_t)b.y * L.pitch + b.x] = moments(f).dr;
+    rho[(int64_t)b.y * L.pitch + b.x] = moments<kSumsOf<T>>(f).dr;
 }
 
 // Fields at the current time t (Eqs. moments, poissonstress, approxdiv).
-template <class W>
+template <int kSums, class W>
 __device__ __forceinline__ void write_fields(float *__restrict__ out, int64_t N, int64_t o,
                                              const float f[9], float sx, float sy, const W &w,
                                              const Lattice &L) {
-    const Mom m = moments(f);
+    const Mom m = moments<kSums>(f);
     const float jx = m.mx + 0.5f * sx, jy = m.my + 0.5f * sy;
     const float rho = L.rho0 + m.dr;
     const float dv = -L.lam_m_mu_r0 * m.dr;
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kBX *kBY) k_fields_interior(const T *__restric
     pull_interior_at<LAY>(src, k, L, f);
     float sx = L.fx, sy = L.fy;
     if (L.grad) source_interior(rho, k, L.pitch, rho[k], L, sx, sy);
-    write_fields(out, N, o, f, sx, sy, uc[k], L);
+    write_fields<kSumsOf<T>>(out, N, o, f, sx, sy, uc[k], L);
 }
 
 template <class T, int LAY = kPull>
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kBB) k_fields_boundary(const T *__restrict__ s
     float sx = L.fx, sy = L.fy;
     if (L.grad) source_boundary(rho, b, k, rho[k], L, sx, sy);
     const int64_t N = (int64_t)L.nx * L.ny, o = (int64_t)b.y * L.nx + b.x;
-    write_fields(out, N, o, f, sx, sy, uc[k], L);
+    write_fields<kSumsOf<T>>(out, N, o, f, sx, sy, uc[k], L);
 }
 
 __global__ void k_advance(int64_t *time, int64_t n) { *time += n; }
@@ -401,7 +401,7 @@ template <class T>
 static void launch_interior(const T *src, T *dst, const DevState &S, const Lattice &L, int toff,
                             cudaStream_t s) {
     if (L.grad) {
-        const dim3 blk(kBX, kGY), grd((L.nx + kBX - 1) / kBX, (L.ny + kGY - 1) / kGY);
+        const dim3 blk(kGX, kGY), grd((L.nx + kGX - 1) / kGX, (L.ny + kGY - 1) / kGY);
         k_interior_grad<T><<<grd, blk, 0, s>>>(src, dst, static_cast<URec<T> *>(S.ucomp), S.cls,
                                                 S.rho, L, S.status,
                                                 S.time, toff);

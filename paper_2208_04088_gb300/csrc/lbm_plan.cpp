@@ -401,15 +401,6 @@ bool tile_plan(const Tables &t, bool wall_node, int shape, TilePlan *p) {
             r.pub0 = (int32_t)p->pubs.size();
             r.link0 = (int32_t)p->links.size();
             const size_t tile = (size_t)ty * ntx + tx;
-            if (first[tile] == first[tile + 1]) {
-                // without boundary nodes a tile holds material or void alone
-                const int x = r.x0 + r.c0, y = r.y0 + r.r0;
-                if (t.cls[(size_t)y * t.pitch + x] == kVoid && !(tx == ntx - 1 && ty == nty - 1 &&
-                                                                p->tiles.empty()))
-                    continue;
-                p->tiles.push_back(r);
-                continue;
-            }
             int count = 0;
             auto publish = [&](int c, int row) {
                 int32_t &s = slot[(size_t)row * W + c];
@@ -458,6 +449,13 @@ bool tile_plan(const Tables &t, bool wall_node, int shape, TilePlan *p) {
             for (size_t k = r.pub0; k < p->pubs.size(); ++k)
                 slot[(size_t)((p->pubs[k] >> 8) & 0xffu) * W + (p->pubs[k] & 0xffu)] = -1;
             if (count > sh.slots()) return false;
+            // without boundary nodes a tile holds material or void alone (an
+            // interior tile: no box edge in its ring); void tiles are left
+            // out, but a lattice without material keeps one, with an empty core
+            if (!count && t.cls[(size_t)(r.y0 + r.r0) * t.pitch + r.x0 + r.c0] == kVoid) {
+                if (tx < ntx - 1 || ty < nty - 1 || !p->tiles.empty()) continue;
+                r.c1 = r.c0;
+            }
             r.npub = (uint16_t)count;
             r.nlink = (uint16_t)(p->links.size() - r.link0);
             p->tiles.push_back(r);
@@ -535,7 +533,10 @@ void tile_choose(const Tables &t, bool grad, bool wall_node, int sms, TilePlan *
     std::vector<std::pair<double, int>> order;
     // from the largest tile down; once a shape fills the SMs several times
     // over, smaller tiles only add halo
-    for (int s = kTileShapeCount - 1; s >= 0; --s) {
+    // (with lambda != mu the densities leave too few registers for four rows to
+    // a thread: 2048^2 in 64 x 64 tiles 121 us a launch of 4 steps, in 64 x 48
+    // 103)
+    for (int s = kTileShapeCount - (grad ? 2 : 1); s >= 0; --s) {
         order.emplace_back(tile_time(t, s, grad, sms), s);
         if ((size_t)ring_count(t.nx, kTileShapes[s].w()) * ring_count(t.ny, kTileShapes[s].h()) >
             (size_t)8 * sms)

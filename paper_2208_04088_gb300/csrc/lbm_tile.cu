@@ -20,11 +20,20 @@
 // boundary path), and the owners pick up the results.  Per node the arithmetic
 // is that of the one-step kernels, so every stored value is bit-identical.
 //
-// What bounds it: FP32 issue in the tiles of a large lattice (a 64 x 64 tile
-// updates 4096 nodes per step, 65 paired operations per pair and 12 per node
-// for the displacement, of which the core's 48 x 48 count); on lattices of
-// less than a few hundred thousand nodes the latency of one step (two block
-// barriers, the collision's and a link's dependent chain) and of the launch.
+// Tiles without boundary nodes (most of a large lattice) take tile_interior:
+// the populations of the block's next tile arrive while this one steps, and the
+// block's warps meet at a split barrier.  Tiles with them take tile_steps.
+//
+// What bounds it: instruction issue in the tiles of a large lattice (a 64 x 64
+// tile updates 4096 nodes per step, 39 paired operations per pair and 7 paired
+// ones per node for the displacement, of which the core's 48 x 48 count; about
+// as many moves, shuffles and address operations go with them).  One interior
+// 64 x 64 tile, 8 steps: 14 us, of which 1.3 us a step (1350 cycles of FP32
+// work in 2740).  On lattices of less than a few hundred thousand nodes it is
+// the latency of one step (two block barriers, the collision's and a link's
+// dependent chain: 2 us in a 32 x 32 tile) and of the launch.  2048^2 edge
+// crack, 500 steps: 12.0 ms (strips 18.9); with lambda != mu 24.8 (one step per
+// launch 45.6); 1024 x 512 plate with a hole, 600 steps: 2.55 (4.25).
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
@@ -61,11 +70,44 @@ template <int LPR, int R> struct Shape {
     static constexpr size_t kOffSlot = ((kStage > kAlias ? kStage : kAlias) + 127) / 128 * 128;
     static constexpr size_t kOffCut = kOffSlot + (size_t)W * H * 2;
     static constexpr size_t kOffU = kOffCut + kSlots;
-    static constexpr size_t kOffBar = kOffU + (size_t)W * H * 16;
-    static constexpr size_t kSmem = kOffBar + 16;
-    static_assert(kSmem <= 232448, "shared memory of one block");
+    static constexpr size_t kEnd = kOffU + (size_t)W * H * 16;
     static_assert(W <= 256 && H <= 256, "copy box");
 };
+
+// Shared memory of a tile without boundary nodes: the populations of the next
+// tile arrive while this one steps, so nothing shares their space; records of
+// the core only; the row exchange in two buffers (one when lambda != mu, whose
+// second barrier per step orders its reuse), and the densities' exchange.
+template <int R, bool GRAD> struct Inner {
+    using S = Shape<32, R>;
+    static constexpr int CW = S::W - 2 * kTileHalo, CH = S::H - 2 * kTileHalo;
+    static constexpr size_t kOffU = S::kStage;
+    static constexpr size_t kOffEx = kOffU + (size_t)CW * CH * 16;
+    static constexpr int kExOne = 2 * (S::G - 1) * 3 * 32;  // words of one buffer
+    static constexpr size_t kOffDen = kOffEx + (size_t)(GRAD ? 1 : 2) * kExOne * 8;
+    static constexpr size_t kEnd = kOffDen + (GRAD ? (size_t)2 * (S::G - 1) * 32 * 8 : 0);
+};
+
+// Barriers and block-wide values, behind the larger of the two layouts.
+struct Control {
+    unsigned long long load, step, den;  // mbarriers: copy landed, rows exchanged, densities exchanged
+    int landed, next;                    // the copy landed in time; the block's next tile
+    TileRec rec;                         // its record
+    float4 *uc;                          // and its displacement records
+    int pitch, pad;
+};
+template <int LPR, int R, bool GRAD> __host__ __device__ constexpr size_t control_at() {
+    if constexpr (LPR == 32)
+        return ((Shape<LPR, R>::kEnd > Inner<R, GRAD>::kEnd ? Shape<LPR, R>::kEnd
+                                                            : Inner<R, GRAD>::kEnd) + 127) / 128 * 128;
+    else
+        return (Shape<LPR, R>::kEnd + 127) / 128 * 128;
+}
+template <int LPR, int R, bool GRAD> constexpr size_t smem_bytes() {
+    static_assert(control_at<LPR, R, GRAD>() + sizeof(Control) + 1024 <= 232448,
+                  "shared memory of one block (with the static part of a batch)");
+    return control_at<LPR, R, GRAD>() + sizeof(Control);
+}
 
 // The pair moved one column to the right (each node takes its left
 // neighbour's value) or to the left.
@@ -110,23 +152,53 @@ __device__ __forceinline__ void wait_for_previous() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// nsteps steps of one tile; the first is step `toff` after *time.
-template <int LPR, int R, bool GRAD>
-__device__ __forceinline__ void tile_steps(const CUtensorMap *tf, float *__restrict__ dst,
+// Copies a tile's populations into the space at the start of shared memory.
+template <int LPR, int R>
+__device__ __forceinline__ void issue_load(const CUtensorMap *tf, const TileRec &rec, uint32_t bar,
+                                           unsigned char *sm) {
+    // order the block's earlier shared-memory accesses before the copy
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    mbar_expect_tx(bar, (uint32_t)Shape<LPR, R>::kStage);
+    tma_load_3d(smem_addr(sm), tf, rec.x0, rec.y0, 0, bar);
+}
+
+// Block-wide wait for the copy; false after the wait limit: the launch is
+// flagged, and the copy waited out so that none is in flight when the block
+// exits.  A limit of 0 gives up at once, whether or not the copy has landed.
+__device__ __forceinline__ bool load_landed(Control *c, uint32_t bar, uint32_t parity,
+                                            const Lattice &L, uint32_t *status) {
+    if (threadIdx.x == 0) {
+        const bool ok = L.wait_ns > 0 && mbar_wait(bar, parity, L.wait_ns);
+        *reinterpret_cast<volatile int *>(&c->landed) = ok;
+        if (!ok) {
+            atomicOr(status, 2u);
+            mbar_wait(bar, parity, kDefaultWaitNs);
+        }
+    }
+    __syncthreads();
+    return *reinterpret_cast<volatile int *>(&c->landed) != 0;
+}
+
+// nsteps steps of one tile, any tile; the first is step `toff` after *time.
+// `first`: the block's first tile (it waits for the previous launch once its
+// tables are read).  Returns false when the copy did not land in time.
+// SRC: the source S is not zero (a body force, or the gradient's).
+template <int LPR, int R, bool GRAD, bool SRC>
+__device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restrict__ dst,
                                            float4 *__restrict__ uc,
                                            const uint8_t *__restrict__ cls, const TileRec &rec,
                                            const uint32_t *__restrict__ pubs,
                                            const TileLink *__restrict__ links,
                                            const BCDev *__restrict__ bcs, const Lattice &L,
                                            const int64_t *__restrict__ time, int toff, int nsteps,
-                                           uint32_t *__restrict__ status, unsigned char *sm) {
+                                           uint32_t *__restrict__ status, unsigned char *sm,
+                                           Control *ctl, bool first, uint32_t load_parity) {
     using S = Shape<LPR, R>;
     constexpr int W = S::W, H = S::H, G = S::G;
     const int tid = threadIdx.x, t = tid % LPR, g = tid / LPR;
     const int c0 = 2 * t, row0 = g * R;
-    const uint32_t bar = smem_addr(sm + S::kOffBar);
+    const uint32_t bar = smem_addr(&ctl->load);
     float4 *us = reinterpret_cast<float4 *>(sm + S::kOffU);
-    volatile int *landed = reinterpret_cast<volatile int *>(sm + S::kOffBar + 8);
 
     // the previous launch writes nothing that is read up to wait_for_previous()
     constexpr uint32_t kNone = 0xffffu;
@@ -152,13 +224,8 @@ __device__ __forceinline__ void tile_steps(const CUtensorMap *tf, float *__restr
             if (__ballot_sync(0xffffffffu, slot[r] != 0xffffffffu)) rowflag |= 1u << r;
         }
     }
-    wait_for_previous();
-    if (tid == 0) {
-        mbar_init(bar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        mbar_expect_tx(bar, (uint32_t)S::kStage);
-        tma_load_3d(smem_addr(sm), tf, rec.x0, rec.y0, 0, bar);
-    }
+    if (first) wait_for_previous();
+    if (tid == 0) issue_load<LPR, R>(tf, rec, bar, sm);
     // while the populations arrive: which of the thread's nodes are material
     // core nodes (bit 2 r + j), and their displacement records
     const float tb0 = (float)(*time + toff - 1);
@@ -179,17 +246,7 @@ __device__ __forceinline__ void tile_steps(const CUtensorMap *tf, float *__restr
 #pragma unroll
     for (int r = 0; r < R; ++r)
         if (__ballot_sync(0xffffffffu, ((mine >> (2 * r)) & 3u) != 0)) corerow |= 1u << r;
-    if (tid == 0)  // a limit of 0 gives up at once, whether or not the copy has landed
-        *landed = L.wait_ns > 0 && mbar_wait(bar, 0, L.wait_ns);
-    __syncthreads();
-    if (!*landed) {
-        // flag it, and keep the block's shared memory until the copy is over
-        if (tid == 0) {
-            atomicOr(status, 2u);
-            mbar_wait(bar, 0, kDefaultWaitNs);
-        }
-        return;
-    }
+    if (!load_landed(ctl, bar, load_parity, L, status)) return false;
     F2 f[R][9];
     {
         const unsigned long long *st = reinterpret_cast<const unsigned long long *>(sm);
@@ -207,7 +264,7 @@ __device__ __forceinline__ void tile_steps(const CUtensorMap *tf, float *__restr
     uint32_t *ruleu = reinterpret_cast<uint32_t *>(rulef);
     constexpr uint32_t kAttrRamp = 1u << 31;
     unsigned long long *den = reinterpret_cast<unsigned long long *>(sm + S::kOffDen);
-    const F2 w2 = splat<F2>(L.omega), s32 = splat<F2>(rmul(L.src, 1.0f / 3.0f));
+    const Relax<F2> rc = relax_of<F2>(L);
     float nonfinite = 0.0f;  // the last step's moments, summed: non-finite if any one is
 
 #pragma unroll 1
@@ -288,10 +345,10 @@ __device__ __forceinline__ void tile_steps(const CUtensorMap *tf, float *__restr
                 const float *gp = pub + own * 12, *yp = pub + ((attr >> 10) & 1023u) * 12;
                 float gx[9];
                 get9(gp, gx);
-                const Mom mx = moments(gx);
+                const Mom mx = moments<kSums32>(gx);
                 float gy[9];
                 get9(yp, gy);
-                const Mom my = moments(gy);
+                const Mom my = moments<kSums32>(gy);
                 // kappa = 0 at a mid-link wall: its upstream population does not count
                 const float gy_i = (flags & kLinkUpstream) ? yp[i] : 0.0f;
                 out[own * 8 + k - 1] =
@@ -358,8 +415,11 @@ __device__ __forceinline__ void tile_steps(const CUtensorMap *tf, float *__restr
             dabove = as_f2(den[(G + (g < G - 1 ? g + 1 : g)) * LPR + t]);
         }
         const bool last = l == nsteps - 1;
+        const int reach = (GRAD ? 2 : 1) * (nsteps - 1 - l);  // rows around the core still needed
 #pragma unroll
         for (int r = 0; r < R; ++r) {
+            if (!__any_sync(0xffffffffu, row0 + r >= rec.r0 - reach && row0 + r < rec.r1 + reach))
+                continue;
             F2 sx = f2(L.fx, L.fx), sy = f2(L.fy, L.fy);
             if constexpr (GRAD) {
                 const F2 rxp = from_right<LPR>(dn[r]), rxm = from_left<LPR>(dn[r]);
@@ -388,7 +448,7 @@ __device__ __forceinline__ void tile_steps(const CUtensorMap *tf, float *__restr
                 }
             }
             F2 dr, jx, jy;
-            collide_v(f[r], sx, sy, w2, s32, dr, jx, jy);
+            collide_sums<SRC>(f[r], sx, sy, rc, dr, jx, jy);
             if ((corerow >> r) & 1u) {
                 // both nodes of every lane, without branches: records of nodes
                 // outside the core are never stored
@@ -432,79 +492,426 @@ __device__ __forceinline__ void tile_steps(const CUtensorMap *tf, float *__restr
         if (m & 2u) uc[k + 1] = us[(2 * r + 1) * kNT + tid];
     }
     if (!isfinite(nonfinite)) flag_nonfinite(status, nonfinite, 0.0f, 0.0f);
+    return true;
 }
 
-template <int LPR, int R, bool GRAD>
+// Two adjacent records (32 bytes, aligned) in one store.
+__device__ __forceinline__ void store_pair_records(float4 *p, const float4 &a, const float4 &b) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y),
+                 "f"(a.z), "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+                 : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void copy16(uint32_t dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// nsteps steps of a tile without boundary nodes (every node of its ring is
+// interior, its core the ring without the halo).  The block's warps meet once
+// per step (twice when lambda != mu) at an mbarrier that they arrive at when
+// their outermost rows are posted and wait at only when they need their
+// neighbours': in between they update their inner rows, so no warp waits for
+// the slowest one's whole step.  Thread 0 takes the block's next tile during
+// the first steps (take_next fills ctl->next, rec, uc, pitch) and copies its
+// populations in behind this tile's; each thread fetches the displacement
+// records of its own nodes of the next tile as soon as those of this one are
+// stored.  early: it does (a launch of too few steps takes the next tile
+// afterwards); loaded: the tile before this one did.
+template <int R, bool GRAD, bool SRC, class Next>
+__device__ __forceinline__ bool tile_interior(const CUtensorMap *tf, float *__restrict__ dst,
+                                              float4 *__restrict__ uc, const TileRec &rec,
+                                              const Lattice &L, int nsteps,
+                                              uint32_t *__restrict__ status, unsigned char *sm,
+                                              Control *ctl, bool first, bool loaded, bool early,
+                                              uint32_t load_parity, uint32_t &phase,
+                                              uint32_t &dphase,
+                                              const Next &take_next) {
+    using S = Shape<32, R>;
+    using I = Inner<R, GRAD>;
+    constexpr int W = S::W, H = S::H, G = S::G, HL = kTileHalo;
+    const int tid = threadIdx.x, t = tid & 31, g = tid >> 5;
+    const int c0 = 2 * t, row0 = g * R;
+    const uint32_t bar = smem_addr(&ctl->load), bstep = smem_addr(&ctl->step), bden = smem_addr(&ctl->den);
+    const bool core = c0 >= HL && c0 < W - HL;  // the core's edges lie between pairs
+    // the thread's record of row r, column c0 + j: [core row][j][core pair]
+    float4 *us = reinterpret_cast<float4 *>(sm + I::kOffU) + (row0 - HL) * I::CW +
+                 (core ? t - HL / 2 : 0);
+    unsigned long long *ex = reinterpret_cast<unsigned long long *>(sm + I::kOffEx);
+    unsigned long long *den = reinterpret_cast<unsigned long long *>(sm + I::kOffDen);
+    auto core_row = [&](int r) { return row0 + r >= HL && row0 + r < H - HL; };  // warp-uniform
+
+    if (first) wait_for_previous();
+    if (tid == 0 && !loaded) issue_load<32, R>(tf, rec, bar, sm);
+    const int64_t k0 = (int64_t)(rec.y0 + row0) * L.pitch + rec.x0 + c0;
+    if (!loaded && core && rec.c1 > rec.c0) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (core_row(r)) {
+                copy16(smem_addr(us + r * I::CW), uc + k0 + (int64_t)r * L.pitch);
+                copy16(smem_addr(us + r * I::CW + I::CW / 2), uc + k0 + (int64_t)r * L.pitch + 1);
+            }
+    }
+    if (!load_landed(ctl, bar, load_parity, L, status)) {
+        copy_wait();
+        return false;
+    }
+    if (rec.c1 == rec.c0) {  // no material in the whole lattice
+        copy_wait();
+        __syncthreads();
+        if (tid == 0 && early)
+            for (int part = 0; part < 3; ++part) take_next(part);
+        __syncthreads();
+        return true;
+    }
+    F2 f[R][9];
+    {
+        // pulled along y by the address (the ring's outermost rows, halo, by
+        // whatever row is there)
+        const unsigned long long *st = reinterpret_cast<const unsigned long long *>(sm);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                int y = row0 + r - c_cy(i);
+                if (r == 0 && c_cy(i) > 0) y = max(y, 0);
+                if (r == R - 1 && c_cy(i) < 0) y = min(y, H - 1);
+                f[r][i] = as_f2(st[((i * H + y) * W + c0) / 2]);
+            }
+    }
+    auto shift_x = [&](int r) {
+        f[r][1] = from_left<32>(f[r][1]);
+        f[r][5] = from_left<32>(f[r][5]);
+        f[r][8] = from_left<32>(f[r][8]);
+        f[r][3] = from_right<32>(f[r][3]);
+        f[r][6] = from_right<32>(f[r][6]);
+        f[r][7] = from_right<32>(f[r][7]);
+    };
+    // the outermost rows to the neighbouring warps
+    auto post = [&](int l) {
+        unsigned long long *eu = ex + (GRAD ? 0 : (l & 1) * I::kExOne) + t, *ed = eu + (G - 1) * 96;
+        if (g < G - 1) {
+            eu[(g * 3 + 0) * 32] = f[R - 1][2].v;
+            eu[(g * 3 + 1) * 32] = f[R - 1][5].v;
+            eu[(g * 3 + 2) * 32] = f[R - 1][6].v;
+        }
+        if (g > 0) {
+            ed[(g * 3 - 3) * 32] = f[0][4].v;
+            ed[(g * 3 - 2) * 32] = f[0][7].v;
+            ed[(g * 3 - 1) * 32] = f[0][8].v;
+        }
+        __syncwarp();
+        if (t == 0) mbar_arrive(bstep);
+    };
+    // rows one up and one down, the outermost from the neighbours
+    auto take = [&](int l) {
+#pragma unroll
+        for (int r = R - 1; r > 0; --r) {
+            f[r][2] = f[r - 1][2];
+            f[r][5] = f[r - 1][5];
+            f[r][6] = f[r - 1][6];
+        }
+#pragma unroll
+        for (int r = 0; r < R - 1; ++r) {
+            f[r][4] = f[r + 1][4];
+            f[r][7] = f[r + 1][7];
+            f[r][8] = f[r + 1][8];
+        }
+        mbar_wait(bstep, phase, kDefaultWaitNs);
+        phase ^= 1;
+        const unsigned long long *eu = ex + (GRAD ? 0 : (l & 1) * I::kExOne) + t, *ed = eu + (G - 1) * 96;
+        if (g > 0) {
+            f[0][2] = as_f2(eu[(g * 3 - 3) * 32]);
+            f[0][5] = as_f2(eu[(g * 3 - 2) * 32]);
+            f[0][6] = as_f2(eu[(g * 3 - 1) * 32]);
+        }
+        if (g < G - 1) {
+            f[R - 1][4] = as_f2(ed[(g * 3 + 0) * 32]);
+            f[R - 1][7] = as_f2(ed[(g * 3 + 1) * 32]);
+            f[R - 1][8] = as_f2(ed[(g * 3 + 2) * 32]);
+        }
+    };
+    const Relax<F2> rc = relax_of<F2>(L);
+    float nonfinite = 0.0f;
+    copy_wait();
+#pragma unroll
+    for (int r = 0; r < R; ++r) shift_x(r);
+    auto step = [&](int l, auto is_last) {
+        constexpr bool last = decltype(is_last)::value;
+        const int reach = (GRAD ? 2 : 1) * (nsteps - 1 - l);  // rows around the core still needed
+        F2 dn[GRAD ? R : 1], dbelow, dabove;
+        if constexpr (GRAD) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) dn[r] = density_of(f[r]);
+            if (g < G - 1) den[g * 32 + t] = dn[R - 1].v;
+            if (g > 0) den[(G - 1 + g - 1) * 32 + t] = dn[0].v;
+            __syncwarp();
+            if (t == 0) mbar_arrive(bden);
+            mbar_wait(bden, dphase, kDefaultWaitNs);
+            dphase ^= 1;
+            dbelow = g > 0 ? as_f2(den[(g - 1) * 32 + t]) : dn[0];
+            dabove = g < G - 1 ? as_f2(den[(G - 1 + g) * 32 + t]) : dn[R - 1];
+        }
+        // the thread's two outermost rows first
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const int r = q == 0 ? 0 : (q == 1 ? R - 1 : q - 1);
+            if (row0 + r >= HL - reach && row0 + r < H - HL + reach) {
+                F2 sx = f2(L.fx, L.fx), sy = f2(L.fy, L.fy);
+                if constexpr (GRAD) {
+                    const F2 ryp = r < R - 1 ? dn[r < R - 1 ? r + 1 : r] : dabove;
+                    const F2 rym = r > 0 ? dn[r > 0 ? r - 1 : 0] : dbelow;
+                    grad_source_open(dn[r], from_right<32>(dn[r]), from_left<32>(dn[r]), ryp, rym, L, sx,
+                                     sy);
+                }
+                F2 dr, jx, jy;
+                collide_sums<SRC>(f[r], sx, sy, rc, dr, jx, jy);
+                if (core_row(r)) {
+                    float dra, drb, jxa, jxb, jya, jyb;
+                    f2_split(dr, dra, drb);
+                    f2_split(jx, jxa, jxb);
+                    f2_split(jy, jya, jyb);
+                    float4 *ua = us + r * I::CW, *ub = ua + I::CW / 2;
+                    float4 wa = *ua, wb = *ub;
+                    integrate_u_value(wa, jxa, jya, L.rho0 + dra);
+                    integrate_u_value(wb, jxb, jyb, L.rho0 + drb);
+                    if (core) {
+                        if (!last) {
+                            *ua = wa;
+                            *ub = wb;
+                        } else {
+                            const int64_t k = k0 + (int64_t)r * L.pitch;
+                            store_pair_records(uc + k, wa, wb);
+                            nonfinite = radd(nonfinite, radd(radd(radd(dra, jxa), jya),
+                                                             radd(radd(drb, jxb), jyb)));
+#pragma unroll
+                            for (int i = 0; i < 9; ++i)
+                                *reinterpret_cast<unsigned long long *>(dst + i * L.fplane + k) = f[r][i].v;
+                            if (early && ctl->next >= 0 && ctl->rec.c1 > ctl->rec.c0) {
+                                const float4 *un =
+                                    ctl->uc + (int64_t)(ctl->rec.y0 + row0 + r) * ctl->pitch + ctl->rec.x0 + c0;
+                                copy16(smem_addr(ua), un);
+                                copy16(smem_addr(ub), un + 1);
+                            }
+                        }
+                    }
+                }
+            }
+            if (q == (R > 1 ? 1 : 0) && !last) {
+                shift_x(0);
+                if (R > 1) shift_x(R - 1);
+                post(l + 1);
+            }
+        }
+        if (!last) {
+#pragma unroll
+            for (int r = 1; r < R - 1; ++r) shift_x(r);
+            take(l + 1);
+        }
+        if (tid == 0 && early) take_next(l);
+    };
+#pragma unroll 1
+    for (int l = 0; l < nsteps - 1; ++l) step(l, std::false_type{});
+    step(nsteps - 1, std::true_type{});
+    if (!isfinite(nonfinite)) flag_nonfinite(status, nonfinite, 0.0f, 0.0f);
+    return true;
+}
+
+// What a launch steps: one lattice, or the instances of a batch (their lattice
+// parameters staged in shared memory when a block turns to another one).
+struct OneLattice {
+    const CUtensorMap *tf;
+    float *out;
+    float4 *u;
+    const uint8_t *classes;
+    const BCDev *bc;
+    const Lattice &l;
+    const int64_t *clock;
+    uint32_t *flags;
+    __device__ void enter(int) {}
+    __device__ const CUtensorMap *map(int) const { return tf; }
+    __device__ float *dst(int) const { return out; }
+    __device__ float4 *uc(int) const { return u; }
+    __device__ int pitch(int) const { return l.pitch; }
+    __device__ const uint8_t *cls(int) const { return classes; }
+    __device__ const BCDev *bcs(int) const { return bc; }
+    __device__ const Lattice &L() const { return l; }
+    __device__ const int64_t *time(int) const { return clock; }
+    __device__ uint32_t *status(int) const { return flags; }
+};
+struct BatchLattices {
+    const TileInst *insts;
+    int cur;
+    Lattice *l;  // shared memory
+    int staged;
+    __device__ void enter(int i) {
+        if (i == staged) return;  // uniform over the block
+        constexpr int kWords = (int)(sizeof(Lattice) / 4);
+        __syncthreads();  // the last tile's reads are over
+        if (threadIdx.x < kWords)
+            reinterpret_cast<uint32_t *>(l)[threadIdx.x] =
+                reinterpret_cast<const uint32_t *>(&insts[i].L)[threadIdx.x];
+        __syncthreads();
+        staged = i;
+    }
+    __device__ const CUtensorMap *map(int i) const { return &insts[i].map[cur]; }
+    __device__ float *dst(int i) const { return insts[i].f[cur ^ 1]; }
+    __device__ float4 *uc(int i) const { return insts[i].uc; }
+    __device__ int pitch(int i) const { return insts[i].L.pitch; }
+    __device__ const uint8_t *cls(int i) const { return insts[i].cls; }
+    __device__ const BCDev *bcs(int i) const { return insts[i].bcs; }
+    __device__ const Lattice &L() const { return *l; }
+    __device__ const int64_t *time(int i) const { return insts[i].time; }
+    __device__ uint32_t *status(int i) const { return insts[i].status; }
+};
+
+// The tiles of a launch.  Tiles of 64 columns are taken by one block per SM,
+// the first by block index and the others from a counter, which the last block
+// to finish puts back to zero; the smallest tiles go one to a block.
+template <int LPR, int R, bool GRAD, bool SRC, class Ctx>
+__device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ tiles, int ntiles,
+                                          int32_t *__restrict__ counter,
+                                          const uint32_t *__restrict__ pubs,
+                                          const TileLink *__restrict__ links, int toff, int nsteps,
+                                          unsigned char *sm) {
+    constexpr size_t kControl = control_at<LPR, R, GRAD>();
+    Control *ctl = reinterpret_cast<Control *>(sm + kControl);
+    release_next();
+    if (threadIdx.x == 0) {
+        mbar_init(smem_addr(&ctl->load), 1);
+        mbar_init(smem_addr(&ctl->step), kNT / 32);
+        mbar_init(smem_addr(&ctl->den), kNT / 32);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    TileRec rec = tiles[blockIdx.x];
+    ctx.enter(rec.inst);
+    if constexpr (LPR != 32) {
+        tile_steps<LPR, R, GRAD, SRC>(ctx.map(rec.inst), ctx.dst(rec.inst), ctx.uc(rec.inst), ctx.cls(rec.inst),
+                                 rec, pubs, links, ctx.bcs(rec.inst), ctx.L(), ctx.time(rec.inst), toff,
+                                 nsteps, ctx.status(rec.inst), sm, ctl, true, 0);
+    } else {
+        const bool more = ntiles > (int)gridDim.x;
+        auto grab = [&]() {
+            const int i = (int)gridDim.x + atomicAdd(counter, 1);
+            return i < ntiles ? i : -1;
+        };
+        // the next tile of an interior one, in three parts a step apart (each
+        // waits for what the one before asked for)
+        auto take_next = [&](int part) {
+            if (part == 0) {
+                ctl->next = more ? grab() : -1;
+            } else if (part == 1 && ctl->next >= 0) {
+                ctl->rec = tiles[ctl->next];
+                issue_load<LPR, R>(ctx.map(ctl->rec.inst), ctl->rec, smem_addr(&ctl->load), sm);
+            } else if (part == 2 && ctl->next >= 0) {
+                ctl->uc = ctx.uc(ctl->rec.inst);
+                ctl->pitch = ctx.pitch(ctl->rec.inst);
+            }
+        };
+        // whether the next tile is known to every thread before this one's last step
+        const bool early = nsteps >= (GRAD ? 4 : 5);
+        bool first = true, loaded = false;
+        uint32_t parity = 0, phase = 0, dphase = 0;
+        for (;;) {
+            bool ok;
+            const int i = rec.inst;
+            const bool ahead = rec.npub == 0 && early;
+            if (rec.npub == 0) {
+                ok = tile_interior<R, GRAD, SRC>(ctx.map(i), ctx.dst(i), ctx.uc(i), rec, ctx.L(), nsteps,
+                                            ctx.status(i), sm, ctl, first, loaded, early, parity, phase,
+                                            dphase, take_next);
+            } else {
+                ok = tile_steps<LPR, R, GRAD, SRC>(ctx.map(i), ctx.dst(i), ctx.uc(i), ctx.cls(i), rec, pubs,
+                                              links, ctx.bcs(i), ctx.L(), ctx.time(i), toff, nsteps,
+                                              ctx.status(i), sm, ctl, first, parity);
+            }
+            if (!ok) break;  // uniform
+            first = false;
+            parity ^= 1;
+            loaded = ahead;
+            if (!ahead) {
+                if (!more) break;
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    ctl->next = grab();
+                    if (ctl->next >= 0) ctl->rec = tiles[ctl->next];
+                }
+                __syncthreads();
+            }
+            if (ctl->next < 0) break;
+            rec = ctl->rec;
+            ctx.enter(rec.inst);
+        }
+        if (more && threadIdx.x == 0 && atomicAdd(counter + 1, 1) == (int)gridDim.x - 1) {
+            counter[0] = 0;
+            counter[1] = 0;
+        }
+    }
+}
+
+template <int LPR, int R, bool GRAD, bool SRC>
 __global__ void __launch_bounds__(kNT, 1)
     k_tile(const __grid_constant__ CUtensorMap tf, float *__restrict__ dst, float4 *__restrict__ uc,
-           const uint8_t *__restrict__ cls, const TileRec *__restrict__ tiles,
-           const uint32_t *__restrict__ pubs, const TileLink *__restrict__ links,
-           const BCDev *__restrict__ bcs, Lattice L, const int64_t *__restrict__ time, int toff,
-           int nsteps, uint32_t *__restrict__ status) {
+           const uint8_t *__restrict__ cls, const TileRec *__restrict__ tiles, int ntiles,
+           int32_t *__restrict__ counter, const uint32_t *__restrict__ pubs,
+           const TileLink *__restrict__ links, const BCDev *__restrict__ bcs,
+           const __grid_constant__ Lattice L, const int64_t *__restrict__ time, int toff, int nsteps,
+           uint32_t *__restrict__ status) {
     extern __shared__ __align__(1024) unsigned char sm[];
-    release_next();
-    const TileRec rec = tiles[blockIdx.x];
-    tile_steps<LPR, R, GRAD>(&tf, dst, uc, cls, rec, pubs, links, bcs, L, time, toff, nsteps, status,
-                             sm);
+    run_tiles<LPR, R, GRAD, SRC>(OneLattice{&tf, dst, uc, cls, bcs, L, time, status}, tiles, ntiles, counter,
+                            pubs, links, toff, nsteps, sm);
 }
 
-// The tiles of many lattices in one launch (a batch, lambda = mu): a tile's
-// instance supplies its buffers, tables and lattice parameters.
-template <int LPR, int R>
+// The tiles of many lattices in one launch (a batch, lambda = mu).
+template <int LPR, int R, bool SRC>
 __global__ void __launch_bounds__(kNT, 1)
-    k_tile_batch(const TileInst *__restrict__ insts, const TileRec *__restrict__ tiles,
-                 const uint32_t *__restrict__ pubs, const TileLink *__restrict__ links, int cur,
-                 int toff, int nsteps) {
+    k_tile_batch(const TileInst *__restrict__ insts, const TileRec *__restrict__ tiles, int ntiles,
+                 int32_t *__restrict__ counter, const uint32_t *__restrict__ pubs,
+                 const TileLink *__restrict__ links, int cur, int toff, int nsteps) {
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(16) Lattice s_L;
-    release_next();
-    const TileRec rec = tiles[blockIdx.x];
-    const TileInst *I = insts + rec.inst;
-    constexpr int kWords = (int)(sizeof(Lattice) / 4);
-    if (threadIdx.x < kWords)
-        reinterpret_cast<uint32_t *>(&s_L)[threadIdx.x] =
-            reinterpret_cast<const uint32_t *>(&I->L)[threadIdx.x];
-    __syncthreads();
-    tile_steps<LPR, R, false>(&I->map[cur], I->f[cur ^ 1], I->uc, I->cls, rec, pubs, links, I->bcs, s_L,
-                              I->time, toff, nsteps, I->status, sm);
+    run_tiles<LPR, R, false, SRC>(BatchLattices{insts, cur, &s_L, -1}, tiles, ntiles, counter, pubs, links,
+                             toff, nsteps, sm);
 }
 
-template <int LPR, int R> cudaError_t batch_shape(const TileBatch &B, int cur, int toff, int nsteps,
-                                                  cudaStream_t s) {
-    static const cudaError_t attr_set = cudaFuncSetAttribute(
-        k_tile_batch<LPR, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Shape<LPR, R>::kSmem);
-    if (attr_set != cudaSuccess || B.ntiles <= 0) return attr_set;
+// One launch of `kernel` over a plan's tiles, in programmatic order.
+template <int LPR, int R, bool GRAD, class... P, class... A>
+cudaError_t launch_tiles(void (*kernel)(P...), int ntiles, int sms, cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)B.ntiles);
+    cfg.gridDim = dim3((unsigned)(LPR == 32 ? std::min(ntiles, sms) : ntiles));
     cfg.blockDim = dim3(kNT);
-    cfg.dynamicSmemBytes = Shape<LPR, R>::kSmem;
+    cfg.dynamicSmemBytes = smem_bytes<LPR, R, GRAD>();
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_tile_batch<LPR, R>, B.insts, B.tiles, B.pubs, B.links, cur, toff,
-                              nsteps);
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-template <int LPR, int R, bool GRAD>
+template <int LPR, int R, bool SRC>
+cudaError_t batch_shape(const TileBatch &B, int cur, int toff, int nsteps, cudaStream_t s) {
+    static const cudaError_t attr_set =
+        cudaFuncSetAttribute(k_tile_batch<LPR, R, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem_bytes<LPR, R, false>());
+    if (attr_set != cudaSuccess || B.ntiles <= 0) return attr_set;
+    return launch_tiles<LPR, R, false>(k_tile_batch<LPR, R, SRC>, B.ntiles, B.sms, s, B.insts, B.tiles,
+                                       B.ntiles, B.counter, B.pubs, B.links, cur, toff, nsteps);
+}
+
+template <int LPR, int R, bool GRAD, bool SRC>
 cudaError_t launch_shape(const Lattice &L, const DevState &S, const TileDev &T, int cur, int toff,
                          int nsteps, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)T.ntiles);
-    cfg.blockDim = dim3(kNT);
-    cfg.dynamicSmemBytes = Shape<LPR, R>::kSmem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_tile<LPR, R, GRAD>, T.map[cur], static_cast<float *>(S.f[cur ^ 1]),
-                              static_cast<float4 *>(S.ucomp), (const uint8_t *)S.cls, T.tiles, T.pubs,
-                              T.links, (const BCDev *)S.bcs, L, (const int64_t *)S.time, toff, nsteps,
-                              S.status);
+    return launch_tiles<LPR, R, GRAD>(k_tile<LPR, R, GRAD, SRC>, T.ntiles, T.sms, s, T.map[cur],
+                                      static_cast<float *>(S.f[cur ^ 1]), static_cast<float4 *>(S.ucomp),
+                                      (const uint8_t *)S.cls, T.tiles, T.ntiles, T.counter, T.pubs, T.links,
+                                      (const BCDev *)S.bcs, L, (const int64_t *)S.time, toff, nsteps,
+                                      S.status);
 }
 
 template <int LPR, int R>
@@ -518,13 +925,16 @@ bool encode_shape(const Lattice &L, const DevState &S, CUtensorMap map[2]) {
     return true;
 }
 
+bool has_force(const Lattice &L) { return L.fx != 0.0f || L.fy != 0.0f; }
+
 template <int LPR, int R> cudaError_t prepare_shape(const Lattice &L, const DevState &S, TileDev *T) {
-    using Sh = Shape<LPR, R>;
     if (!encode_shape<LPR, R>(L, S, T->map)) return cudaErrorInvalidValue;
-    return L.grad ? cudaFuncSetAttribute(k_tile<LPR, R, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::kSmem)
-                  : cudaFuncSetAttribute(k_tile<LPR, R, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::kSmem);
+    auto limit = [](auto kernel, size_t bytes) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    if (L.grad) return limit(k_tile<LPR, R, true, true>, smem_bytes<LPR, R, true>());
+    return has_force(L) ? limit(k_tile<LPR, R, false, true>, smem_bytes<LPR, R, false>())
+                        : limit(k_tile<LPR, R, false, false>, smem_bytes<LPR, R, false>());
 }
 
 }  // namespace
@@ -544,8 +954,9 @@ cudaError_t launch_tile(const Lattice &L, const DevState &S, const TileDev &T, i
                         int nsteps, cudaStream_t s) {
 #define LBM_TILE(n, lpr, r)                                                                  \
     case n:                                                                                  \
-        return L.grad ? launch_shape<lpr, r, true>(L, S, T, cur, toff, nsteps, s)            \
-                      : launch_shape<lpr, r, false>(L, S, T, cur, toff, nsteps, s);
+        return L.grad         ? launch_shape<lpr, r, true, true>(L, S, T, cur, toff, nsteps, s)  \
+               : has_force(L) ? launch_shape<lpr, r, false, true>(L, S, T, cur, toff, nsteps, s) \
+                              : launch_shape<lpr, r, false, false>(L, S, T, cur, toff, nsteps, s);
     switch (T.shape) {
         LBM_TILE(0, 16, 1)
         LBM_TILE(1, 32, 2)
@@ -566,12 +977,18 @@ bool tile_maps(const Lattice &L, const DevState &S, int shape, CUtensorMap map[2
 }
 
 cudaError_t launch_tile_batch(const TileBatch &B, int cur, int toff, int nsteps, cudaStream_t s) {
+#define LBM_TILE(n, lpr, r)                                                  \
+    case n:                                                                  \
+        return B.force ? batch_shape<lpr, r, true>(B, cur, toff, nsteps, s)  \
+                       : batch_shape<lpr, r, false>(B, cur, toff, nsteps, s);
     switch (B.shape) {
-        case 0: return batch_shape<16, 1>(B, cur, toff, nsteps, s);
-        case 1: return batch_shape<32, 2>(B, cur, toff, nsteps, s);
-        case 2: return batch_shape<32, 3>(B, cur, toff, nsteps, s);
-        default: return batch_shape<32, 4>(B, cur, toff, nsteps, s);
+        LBM_TILE(0, 16, 1)
+        LBM_TILE(1, 32, 2)
+        LBM_TILE(2, 32, 3)
+        LBM_TILE(3, 32, 4)
     }
+#undef LBM_TILE
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace lbm

@@ -167,7 +167,7 @@ __device__ __forceinline__ void wave_region(
     const int nsweep = Hs + 3 * kK - 3;
     const float tb = (float)(*time + toff + lv - 2);  // boundary data at the time of f^col
     const F2 sx2 = f2(L.fx, L.fx), sy2 = f2(L.fy, L.fy);
-    const F2 w2 = splat<F2>(L.omega), s32 = splat<F2>(rmul(L.src, 1.0f / 3.0f));
+    const Relax<F2> rc = relax_of<F2>(L);
 
     auto issue = [&](int j) {
         const uint32_t bar = bar0 + 8u * (uint32_t)(j & (kNI - 1));
@@ -293,12 +293,12 @@ __device__ __forceinline__ void wave_region(
                                 const BLink *lrec = blinks + boundary_index(wb, L) * 8;
                                 auto link = [&](int i) { return simple ? sl : lrec[i - 1]; };
                                 float f0;
-                                const float fk = boundary8_pull(
+                                const float fk = boundary8_pull<kSums32>(
                                     Rows{rm - c, r0 - c, rp - c, cb}, nw_mask(wb, 2), nw_mask(wb, 10),
                                     nw_mask(wb, 18), nw_mask(wb, 26), kdir, link, bcs, tb, L, f0);
                                 float fr, jx, jy, m00;
                                 const float mine =
-                                    boundary8_collide(fk, f0, kdir, L.fx, L.fy, L, fr, jx, jy, m00);
+                                    boundary8_collide<kSums32>(fk, f0, kdir, L.fx, L.fy, L, fr, jx, jy, m00);
                                 if (live) {
                                     const int64_t gb = (int64_t)y * L.pitch + xin + cb;
                                     if (lv < kK) {
@@ -350,7 +350,7 @@ __device__ __forceinline__ void wave_region(
                                 const int dc = h << 5;
                                 if (h ? sim_b : sim_a) {
                                     const uint64_t wn = h ? nwb : nwa;
-                                    simple_pull<false>(
+                                    simple_pull<false, kSums32>(
                                         Rows{rm - c, r0 - c, rp - c, c + dc}, nw_mask(wn, 2),
                                         nw_mask(wn, 10), nw_mask(wn, 26),
                                         simple_link((uint32_t)(wn >> 35), L), bcs, tb, L, g);
@@ -374,7 +374,7 @@ __device__ __forceinline__ void wave_region(
                             }
                         }
                         F2 dr, jx, jy;
-                        collide_v(f, sx2, sy2, w2, s32, dr, jx, jy);
+                        collide_sums<true>(f, sx2, sy2, rc, dr, jx, jy);
                         if (lv < kK)
                             store_pair(own, kC, f, do_a, do_b);
                         else
@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(kGradThreads, 1)
     const int j_last = Hs + 4 * kGradK - 1;
     const int nsweep = Hs + 6 * kGradK - 3;
     const float tb = (float)(*time + toff + lv - 2);  // boundary data at the time of f^col
-    const F2 w2 = splat<F2>(L.omega), s32 = splat<F2>(rmul(L.src, 1.0f / 3.0f));
+    const Relax<F2> rc = relax_of<F2>(L);
 
     auto issue = [&](int j) {
         const uint32_t bar = bar0 + 8u * (uint32_t)(j & (kGradNI - 1));
@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(kGradThreads, 1)
                 const int dc = h << 5;
                 if (h ? sim_b : sim_a) {
                     const uint64_t wn = h ? nwb : nwa;
-                    simple_pull<false>(Rows{rm - c, r0 - c, rp - c, c + dc}, nw_mask(wn, 2),
+                    simple_pull<false, kSums32>(Rows{rm - c, r0 - c, rp - c, c + dc}, nw_mask(wn, 2),
                                        nw_mask(wn, 10), nw_mask(wn, 26),
                                        simple_link((uint32_t)(wn >> 35), L), bcs, tb, L, g);
                 } else {
@@ -656,7 +656,7 @@ __global__ void __launch_bounds__(kGradThreads, 1)
             const BLink *lrec = blinks + boundary_index(wb, L) * 8;
             auto link = [&](int i) { return lrec[i - 1]; };
             float g0, f[9];
-            const float fk = boundary8_pull(Rows{rm - c, r0 - c, rp - c, cb}, nw_mask(wb, 2),
+            const float fk = boundary8_pull<kSums32>(Rows{rm - c, r0 - c, rp - c, cb}, nw_mask(wb, 2),
                                             nw_mask(wb, 10), nw_mask(wb, 18), nw_mask(wb, 26),
                                             kdir, link, bcs, tb, L, g0);
             gather8(fk, g0, f);
@@ -756,7 +756,7 @@ __global__ void __launch_bounds__(kGradThreads, 1)
                                nwa, nwb, [&](float *f, int cb, uint64_t wb, bool live) {
                                    float sx, sy, dr, jx, jy;
                                    source_one(f, cb, wb, false, sx, sy);
-                                   collide(f, sx, sy, L, dr, jx, jy);
+                                   collide<kSums32>(f, sx, sy, L, dr, jx, jy);
                                    float mine = f[1];
 #pragma unroll
                                    for (int q = 2; q < 9; ++q)
@@ -806,7 +806,7 @@ __global__ void __launch_bounds__(kGradThreads, 1)
                             sy = f2(sya, syb);
                         }
                         F2 dr, jx, jy;
-                        collide_v(f, sx, sy, w2, s32, dr, jx, jy);
+                        collide_sums<true>(f, sx, sy, rc, dr, jx, jy);
                         if (lv < kGradK)
                             store_pair(own + c, kC, f, do_a, do_b);
                         else
