@@ -78,12 +78,12 @@ constexpr int kTileRun = 4;
 // adjacent nodes (interior_pair), and a tile of TX x TY threads covers
 // 2 TX x TY nodes.  Threads per SM the register bound allows: on 256 plates
 // with a hole, FP16 measured 79.6 GLUPS at 1536 (40 registers), 79.4 at 1280,
-// 76.4 at 1024; BF16 78.7, 81.7 and 78.5.
+// 76.4 at 1024; BF16 78.7, 81.7 and 78.5.  40 FP16 plates in runs of four 32 x 4
+// tiles: 41.7 ms for 256 steps at 1280, 42.2 at 1536.
 template <class T, bool kMixed>
 constexpr bool kBatchPair = !kMixed && !std::is_same<T, float>::value;
 template <class T, bool kMixed>
-constexpr int kBatchThreadsPerSm =
-    !kBatchPair<T, kMixed> ? 2048 : (std::is_same<T, __half>::value ? 1536 : 1280);
+constexpr int kBatchThreadsPerSm = kBatchPair<T, kMixed> ? 1280 : 2048;
 
 template <class T, int TX, int TY, bool kMixed>
 __global__ void __launch_bounds__(TX *TY, kBatchThreadsPerSm<T, kMixed> / (TX * TY)) k_batch_interior(const InstDev *__restrict__ insts,
@@ -1100,6 +1100,12 @@ extern "C" lbm_status lbm_batch_create(const lbm_desc *descs, int32_t count, voi
     std::unique_ptr<lbm_engine> E(new lbm_engine());
     lbm_status st = engine_init(E.get(), descs[0].storage, stream);
     if (st != LBM_OK) return st;
+    // A lockstep batch keeps its tiles, so its grid can follow them: runs of
+    // four small tiles per block stage an instance's descriptor once per run
+    // and leave the order to the block scheduler (40 FP16 plates with holes,
+    // 256 steps: 42.3 ms; 46.8 with one tile per block, 50.7 with the
+    // persistent grid, which the server keeps).
+    E->shape = {32, 4, 16, 3};
     uint64_t total = 0;
     for (int32_t i = 0; i < count; ++i) {
         uint64_t b = 0;

@@ -27,7 +27,10 @@
 namespace lbm {
 // ---------------------------------------------------------------------------
 // Kernels.
-constexpr int kBX = 32, kBY = 8;
+// Blocks of 128 x 2 threads: one step in place of the 2048^2 crack 74.5 us, with
+// 64 x 4 75.0, with 32 x 8 76.4 (a block then touches fewer, longer runs of
+// every population plane).
+constexpr int kBX = 128, kBY = 2;
 constexpr int kBB = 64;  // threads per block of the boundary-list kernels
 
 // Interior kernel: one node per thread (NR rows per thread, kBY rows apart).
@@ -68,13 +71,17 @@ __global__ void __launch_bounds__(kBX *kBY, 8) k_interior(const T *src, T *dst,
 }
 
 // 16-bit storage, two buffers, lambda = mu: two adjacent nodes per thread
-// (interior_pair).  Blocks per SM the register bound aims at: FP16 measured fastest at six (40
-// registers: 93.9 against 90.4 GLUPS at four on the 2048^2 crack), BF16 at four
-// (100.7 against 98.9 at six).
-template <class T> constexpr int kPairMinBlocks = std::is_same<T, __half>::value ? 6 : 4;
+// (interior_pair).  Threads per SM the register bound aims at: FP16 measured fastest at 1536 (40
+// registers: 93.9 against 90.4 GLUPS at 1024 on the 2048^2 crack), BF16 at 1024
+// (100.7 against 98.9 at 1536).  Blocks of 64 threads in one row: 21.6 ms for
+// 500 steps of the FP16 crack, 21.9 with 128, 22.5 with 128 x 2, 23.0 with
+// 32 x 8 (longer runs of every plane, and the next block placed as soon as two
+// warps end).
+template <class T> constexpr int kPairMinBlocks = std::is_same<T, __half>::value ? 24 : 16;
+constexpr int kPX = 64;  // threads of its blocks, all in one row
 
 template <class T>
-__global__ void __launch_bounds__(kBX *kBY, kPairMinBlocks<T>) k_interior_pair(const T *__restrict__ src,
+__global__ void __launch_bounds__(kPX, kPairMinBlocks<T>) k_interior_pair(const T *__restrict__ src,
                                                             T *__restrict__ dst,
                                                             float2 *__restrict__ uc,
                                                             const uint8_t *__restrict__ cls,
@@ -82,8 +89,8 @@ __global__ void __launch_bounds__(kBX *kBY, kPairMinBlocks<T>) k_interior_pair(c
                                                             uint32_t *__restrict__ status,
                                                             const int64_t *__restrict__ time,
                                                             int toff) {
-    const int x0 = 2 * (int)(blockIdx.x * kBX + threadIdx.x);
-    const int y = blockIdx.y * kBY + threadIdx.y;
+    const int x0 = 2 * (int)(blockIdx.x * kPX + threadIdx.x);
+    const int y = blockIdx.y + threadIdx.y;  // threadIdx.y = 0
     // FP16: this step's scales.  The thread of node (0, 0), which is never
     // interior, publishes them after its node classes have been read, so that
     // no store sits between the loads of a thread and delays them.
@@ -409,8 +416,8 @@ static void launch_interior(const T *src, T *dst, const DevState &S, const Latti
     }
     if constexpr (!std::is_same<T, float>::value) {
         // 16-bit storage: two nodes per thread
-        const dim3 blk(kBX, kBY), grd((L.nx + 2 * kBX - 1) / (2 * kBX), (L.ny + kBY - 1) / kBY);
-        k_interior_pair<T><<<grd, blk, 0, s>>>(src, dst, static_cast<float2 *>(S.ucomp), S.cls, L,
+        const dim3 grd((L.nx + 2 * kPX - 1) / (2 * kPX), L.ny);
+        k_interior_pair<T><<<grd, kPX, 0, s>>>(src, dst, static_cast<float2 *>(S.ucomp), S.cls, L,
                                                S.status, S.time, toff);
         return;
     }
