@@ -143,6 +143,22 @@ __device__ __forceinline__ void get9(const float *p, float v[9]) {
     v[8] = p[8];
 }
 
+// The rule of a tile's link at boundary time tb, and its attributes: slots of
+// its node and of the upstream node (the node itself if it is not read),
+// direction it arrives in, flags, and whether its data change with time.
+constexpr uint32_t kAttrRamp = 1u << 31;
+__device__ __forceinline__ LinkRule make_rule(const TileLink &lk, const BCDev *__restrict__ bcs,
+                                              float tb, const Lattice &L, uint32_t &attr) {
+    const int i = lk.dir, k = i <= 4 ? (i + 1) % 4 + 1 : (i - 3) % 4 + 5;
+    const BLink b{lk.q, lk.n0, lk.n1, lk.bc, lk.bc2};
+    attr = lk.own | (uint32_t)((lk.flags & kLinkUpstream) ? lk.up : lk.own) << 10 | (uint32_t)k << 20 |
+           (uint32_t)lk.flags << 24;
+    if (bcs[lk.bc].profile == LBM_PROFILE_RAMP || bcs[lk.bc2].profile == LBM_PROFILE_RAMP)
+        attr |= kAttrRamp;
+    return link_rule(k, lk.flags & kLinkMiss, lk.flags & kLinkDirichlet, lk.flags & kLinkCorner, b, bcs,
+                     tb, L);
+}
+
 // Programmatic launch order: the next launch of the stream may start its
 // prologue now, and this one has waited for everything before it.
 __device__ __forceinline__ void release_next() {
@@ -200,32 +216,59 @@ __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restr
     const uint32_t bar = smem_addr(&ctl->load);
     float4 *us = reinterpret_cast<float4 *>(sm + S::kOffU);
 
-    // the previous launch writes nothing that is read up to wait_for_previous()
+    // the previous launch writes nothing that is read before wait_for_previous()
     constexpr uint32_t kNone = 0xffffu;
     const int npub = rec.npub, nlink = rec.nlink;
+    // The rule of the thread's (first) link stays in registers where the tile
+    // leaves room for it, in shared memory otherwise (350 cycles a step).
+    constexpr bool kKeep = R == 1 || (R == 2 && !GRAD);
+    // cut masks in registers likewise
+    constexpr bool kCuts = !GRAD || R <= 2;
     uint8_t *cutm = sm + S::kOffCut;
     uint32_t slot[R];       // slots of the thread's published nodes (low, high half)
+    uint32_t cuts[(R + 1) / 2];  // their cut masks, a byte per node (kCuts)
     uint32_t rowflag = 0;   // rows in which a lane of the warp has one (warp-uniform)
 #pragma unroll
     for (int r = 0; r < R; ++r) slot[r] = 0xffffffffu;
+#pragma unroll
+    for (int r = 0; r < (R + 1) / 2; ++r) cuts[r] = 0;
+    // The last warp starts the copy (in a block's first tile once the previous
+    // launch is over) while the others read the tile's tables.
+    constexpr int kReaders = kNT - 32;
+    if (tid == kReaders) {
+        if (first) wait_for_previous();
+        issue_load<LPR, R>(tf, rec, bar, sm);
+    }
     if (npub) {  // uniform over the block
         uint32_t *map = reinterpret_cast<uint32_t *>(sm + S::kOffSlot);
-        for (int q = tid; q < W * H / 2; q += kNT) map[q] = 0xffffffffu;
-        __syncthreads();
-        for (int q = tid; q < npub; q += kNT) {
-            const uint32_t p = pubs[rec.pub0 + q];
-            reinterpret_cast<uint16_t *>(map)[((p >> 8) & 0xffu) * W + (p & 0xffu)] = (uint16_t)q;
-            cutm[q] = (uint8_t)(p >> 16);
+        if (tid < kReaders) {
+            for (int q = tid; q < W * H / 2; q += kReaders) map[q] = 0xffffffffu;
+            asm volatile("barrier.cta.sync 1, %0;" ::"n"(kReaders) : "memory");
+            for (int q = tid; q < npub; q += kReaders) {
+                const uint32_t p = pubs[rec.pub0 + q];
+                reinterpret_cast<uint16_t *>(map)[((p >> 8) & 0xffu) * W + (p & 0xffu)] = (uint16_t)q;
+                cutm[q] = (uint8_t)(p >> 16);
+            }
         }
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             slot[r] = map[((row0 + r) * W + c0) / 2];
+            const uint32_t sa = slot[r] & 0xffffu, sb = slot[r] >> 16;
+            if (kCuts) cuts[r / 2] |= ((sa != kNone ? cutm[sa] : 0u) | (sb != kNone ? cutm[sb] : 0u) << 8)
+                           << (16 * (r & 1));
             if (__ballot_sync(0xffffffffu, slot[r] != 0xffffffffu)) rowflag |= 1u << r;
         }
     }
+    // the cut masks of row r's two nodes
+    auto cut_masks = [&](int r) -> uint32_t {
+        if (kCuts) return cuts[r / 2] >> (16 * (r & 1));
+        const uint32_t sa = slot[r] & 0xffffu, sb = slot[r] >> 16;
+        return (sa != kNone ? cutm[sa] : 0u) | (sb != kNone ? cutm[sb] : 0u) << 8;
+    };
+    TileLink my_link;
+    if (kKeep && tid < nlink) my_link = links[rec.link0 + tid];
     if (first) wait_for_previous();
-    if (tid == 0) issue_load<LPR, R>(tf, rec, bar, sm);
     // while the populations arrive: which of the thread's nodes are material
     // core nodes (bit 2 r + j), and their displacement records
     const float tb0 = (float)(*time + toff - 1);
@@ -246,6 +289,9 @@ __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restr
 #pragma unroll
     for (int r = 0; r < R; ++r)
         if (__ballot_sync(0xffffffffu, ((mine >> (2 * r)) & 3u) != 0)) corerow |= 1u << r;
+    uint32_t my_attr = 0;
+    LinkRule my_rule{};
+    if (kKeep && tid < nlink) my_rule = make_rule(my_link, bcs, tb0, L, my_attr);
     if (!load_landed(ctl, bar, load_parity, L, status)) return false;
     F2 f[R][9];
     {
@@ -262,7 +308,6 @@ __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restr
     float *out = reinterpret_cast<float *>(sm + S::kOffOut);
     float *rulef = reinterpret_cast<float *>(sm + S::kOffRule);  // [9][kRules]: attributes, LinkRule
     uint32_t *ruleu = reinterpret_cast<uint32_t *>(rulef);
-    constexpr uint32_t kAttrRamp = 1u << 31;
     unsigned long long *den = reinterpret_cast<unsigned long long *>(sm + S::kOffDen);
     const Relax<F2> rc = relax_of<F2>(L);
     float nonfinite = 0.0f;  // the last step's moments, summed: non-finite if any one is
@@ -309,32 +354,26 @@ __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restr
             const float tb = tb0 + (float)l;  // boundary data at the time of f^col
 #pragma unroll 1
             for (int e = tid; e < nlink; e += kNT) {
-                uint32_t attr;
-                LinkRule rule;
-                bool fresh = l == 0 || tb == 0.0f || e >= S::kRules;
+                uint32_t attr = my_attr;
+                LinkRule rule = my_rule;
+                const bool mine_kept = kKeep && e == tid;
+                bool fresh = tb == 0.0f || (!mine_kept && (l == 0 || e >= S::kRules));
                 if (!fresh) {
-                    attr = ruleu[e];
+                    if (!mine_kept) attr = ruleu[e];
                     fresh = (attr & kAttrRamp) != 0;
                 }
                 if (fresh) {
-                    const TileLink lk = links[rec.link0 + e];
-                    const int i = lk.dir, kk = i <= 4 ? (i + 1) % 4 + 1 : (i - 3) % 4 + 5;
-                    const BLink b{lk.q, lk.n0, lk.n1, lk.bc, lk.bc2};
-                    // slots, direction, flags (an upstream node not read: the node itself)
-                    attr = lk.own | (uint32_t)((lk.flags & kLinkUpstream) ? lk.up : lk.own) << 10 |
-                           (uint32_t)kk << 20 | (uint32_t)lk.flags << 24;
-                    if (bcs[lk.bc].profile == LBM_PROFILE_RAMP || bcs[lk.bc2].profile == LBM_PROFILE_RAMP)
-                        attr |= kAttrRamp;
-                    rule = link_rule(kk, lk.flags & kLinkMiss, lk.flags & kLinkDirichlet,
-                                     lk.flags & kLinkCorner, b, bcs, tb, L);
-                    if (e < S::kRules) {
+                    rule = make_rule(links[rec.link0 + e], bcs, tb, L, attr);
+                    if (mine_kept) {
+                        my_rule = rule;
+                    } else if (e < S::kRules) {
                         ruleu[e] = attr;
                         const float v[8] = {rule.q, rule.kap, rule.fac, rule.t0,
                                             rule.t1, rule.c0, rule.c1, rule.c2};
 #pragma unroll
                         for (int m = 0; m < 8; ++m) rulef[(1 + m) * S::kRules + e] = v[m];
                     }
-                } else {
+                } else if (!mine_kept) {
                     float v[8];
 #pragma unroll
                     for (int m = 0; m < 8; ++m) v[m] = rulef[(1 + m) * S::kRules + e];
@@ -387,7 +426,7 @@ __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restr
                 if (!((rowflag >> r) & 1u)) continue;
                 const uint32_t sa = slot[r] & 0xffffu, sb = slot[r] >> 16;
                 // every lane reads (slot 0 where it has none): no lane waits for another
-                const uint32_t ca = sa != kNone ? cutm[sa] : 0u, cb = sb != kNone ? cutm[sb] : 0u;
+                const uint32_t ca = cut_masks(r), cb = ca >> 8;
                 const float4 *oa = reinterpret_cast<const float4 *>(out + (sa != kNone ? sa : 0u) * 8);
                 const float4 *ob = reinterpret_cast<const float4 *>(out + (sb != kNone ? sb : 0u) * 8);
                 const float4 a0 = oa[0], a1 = oa[1], b0 = ob[0], b1 = ob[1];
@@ -427,8 +466,7 @@ __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restr
                 const F2 rym = r > 0 ? dn[r > 0 ? r - 1 : 0] : dbelow;
                 if ((rowflag >> r) & 1u) {
                     // one-sided where an axis neighbour is across a wall
-                    const uint32_t sa = slot[r] & 0xffffu, sb = slot[r] >> 16;
-                    const uint32_t ca = sa != kNone ? cutm[sa] : 0u, cb = sb != kNone ? cutm[sb] : 0u;
+                    const uint32_t ca = cut_masks(r), cb = ca >> 8;
                     float d[2], xp[2], xm[2], yp[2], ym[2], hx[2], hy[2];
                     f2_split(dn[r], d[0], d[1]);
                     f2_split(rxp, xp[0], xp[1]);
@@ -932,7 +970,9 @@ template <int LPR, int R> cudaError_t prepare_shape(const Lattice &L, const DevS
     auto limit = [](auto kernel, size_t bytes) {
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
-    if (L.grad) return limit(k_tile<LPR, R, true, true>, smem_bytes<LPR, R, true>());
+    if constexpr (R < 4)
+        if (L.grad) return limit(k_tile<LPR, R, true, true>, smem_bytes<LPR, R, true>());
+    if (L.grad) return cudaErrorInvalidValue;
     return has_force(L) ? limit(k_tile<LPR, R, false, true>, smem_bytes<LPR, R, false>())
                         : limit(k_tile<LPR, R, false, false>, smem_bytes<LPR, R, false>());
 }
@@ -952,11 +992,14 @@ cudaError_t tile_prepare(const Lattice &L, const DevState &S, TileDev *T) {
 
 cudaError_t launch_tile(const Lattice &L, const DevState &S, const TileDev &T, int cur, int toff,
                         int nsteps, cudaStream_t s) {
-#define LBM_TILE(n, lpr, r)                                                                  \
-    case n:                                                                                  \
-        return L.grad         ? launch_shape<lpr, r, true, true>(L, S, T, cur, toff, nsteps, s)  \
-               : has_force(L) ? launch_shape<lpr, r, false, true>(L, S, T, cur, toff, nsteps, s) \
-                              : launch_shape<lpr, r, false, false>(L, S, T, cur, toff, nsteps, s);
+    // the plans with lambda != mu take no tile of four rows to a thread
+#define LBM_TILE(n, lpr, r)                                                                      \
+    case n:                                                                                      \
+        if constexpr (r < 4)                                                                     \
+            if (L.grad) return launch_shape<lpr, r, true, true>(L, S, T, cur, toff, nsteps, s);  \
+        if (L.grad) break;                                                                       \
+        return has_force(L) ? launch_shape<lpr, r, false, true>(L, S, T, cur, toff, nsteps, s)   \
+                            : launch_shape<lpr, r, false, false>(L, S, T, cur, toff, nsteps, s);
     switch (T.shape) {
         LBM_TILE(0, 16, 1)
         LBM_TILE(1, 32, 2)
