@@ -541,8 +541,7 @@ lbm_status build_tile_tables(lbm_engine *E) {
         }
         if (ok) break;  // the smallest tiles always are
     }
-    std::stable_sort(all.tiles.begin(), all.tiles.end(),
-                     [](const TileRec &a, const TileRec &b) { return a.nlink > b.nlink; });
+    tile_sort(all.tiles);
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     const size_t bi = up(sizeof(TileInst) * inst.size()), bt = up(sizeof(TileRec) * all.tiles.size());
     const size_t bp = up(sizeof(uint32_t) * all.pubs.size()), bl = up(sizeof(TileLink) * all.links.size());
@@ -560,6 +559,7 @@ lbm_status build_tile_tables(lbm_engine *E) {
     // sets the kernel's shared-memory limit (outside any capture); launches nothing
     e = launch_tile_batch(E->tile, 0, 0, 0, E->stream);
     E->tile.ntiles = (int)all.tiles.size();
+    E->tile.nrules = tile_rules(all, E->tile.sms);
     E->nblocked = (int)inst.size();
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(m, inst.data(), sizeof(TileInst) * inst.size(), cudaMemcpyHostToDevice,
@@ -824,6 +824,7 @@ lbm_status engine_steps(lbm_engine *E, int64_t nsteps) {
     int64_t done = 0;
     // boundary, simple boundary nodes, interior, advance (+ scatter with in-place instances)
     const int per_step = one_step_instances(E) > 0 ? (E->n_in_place > 0 ? 5 : 4) : 0;
+    const int kernels = E->tile.nrules > 0 ? 2 : 1;  // of a launch of the tiles
     if (nsteps >= kChunk) {
         if (!E->graph[E->wcur]) {
             lbm_status st = build_batch_graph(E);
@@ -832,7 +833,7 @@ lbm_status engine_steps(lbm_engine *E, int64_t nsteps) {
         for (; done + kChunk <= nsteps; done += kChunk) {
             e = cudaGraphLaunch(E->graph[E->wcur], E->stream);
             if (e != cudaSuccess) return fail_cuda(e, "batch: graph launch");
-            E->launches += per_step * kChunk + (E->nblocked > 0 ? kChunk / kWaveK + 1 : 0);
+            E->launches += per_step * kChunk + (E->nblocked > 0 ? kChunk / kWaveK * kernels + 1 : 0);
         }
     }
     const int64_t rest = nsteps - done;
@@ -846,7 +847,7 @@ lbm_status engine_steps(lbm_engine *E, int64_t nsteps) {
         if (E->nblocked > 0) {
             e = launch_blocked(E, rest, &E->wcur, E->stream);
             if (e != cudaSuccess) return fail_cuda(e, "batch: tile launch");
-            E->launches += (rest + kWaveK - 1) / kWaveK + 1;
+            E->launches += (rest + kWaveK - 1) / kWaveK * kernels + 1;
         }
     }
     E->step_count += nsteps;

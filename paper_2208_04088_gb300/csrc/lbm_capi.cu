@@ -179,6 +179,10 @@ cudaError_t launch_blocked(lbm_solver *h, int cur, int toff, int nsteps, cudaStr
                               : launch_wave(h->L, h->S, h->wave, cur, toff, s);
 }
 
+int kernels_per_blocked(const lbm_solver *h) {
+    return h->tile.shape >= 0 && h->tile.nrules > 0 ? 2 : 1;
+}
+
 lbm_status build_graph(lbm_solver *h, int start) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(h->cap_main, cudaStreamCaptureModeThreadLocal);
@@ -284,6 +288,7 @@ static cudaError_t tile_create(lbm_solver *h) {
     T.ntiles = (int)plan.tiles.size();
     T.shape = plan.shape;
     T.sms = device_sms();
+    T.nrules = tile_rules(plan, T.sms);
     // pageable sources: the copies are staged before the calls return
     cudaError_t e = cudaMemcpyAsync(m, plan.tiles.data(), plan.tiles.size() * sizeof(TileRec),
                                     cudaMemcpyHostToDevice, h->stream);
@@ -497,7 +502,7 @@ extern "C" lbm_status lbm_step(lbm_handle h, int64_t nsteps) {
                 if (e == cudaSuccess) e = cudaEventRecord(ev.before_boundary, h->stream);
                 if (e == cudaSuccess) e = cudaEventRecord(ev.after_boundary, h->stream);
                 s += h->block - 1;
-                h->launches += 1;
+                h->launches += kernels_per_blocked(h);
             } else {
                 e = launch_step(h->storage, h->L, h->S, h->cur, (int)s, h->stream, h->cap_side,
                                 h->fork, h->join, &ev);
@@ -517,7 +522,8 @@ extern "C" lbm_status lbm_step(lbm_handle h, int64_t nsteps) {
             }
             e = cudaGraphLaunch(h->graph[h->cur], h->stream);
             if (e != cudaSuccess) return cuda_fail(e, "lbm_step: graph launch");
-            h->launches += (h->block > 1 ? kGraphChunk / h->block : kGraphChunk * per_step) + 1;
+            h->launches += (h->block > 1 ? kGraphChunk / h->block * kernels_per_blocked(h)
+                                         : kGraphChunk * per_step) + 1;
         }
     }
     const int64_t rest = nsteps - done;
@@ -526,7 +532,7 @@ extern "C" lbm_status lbm_step(lbm_handle h, int64_t nsteps) {
         if (h->block > 1 && (n == h->block || (h->tile.shape >= 0 && n >= kTileMinSteps))) {
             e = launch_blocked(h, h->cur, (int)s, n, h->stream);
             s += n;
-            h->launches += 1;
+            h->launches += kernels_per_blocked(h);
         } else {
             e = launch_step(h->storage, h->L, h->S, h->cur, (int)s, h->stream, nullptr, nullptr,
                             nullptr, nullptr);

@@ -293,6 +293,16 @@ struct TilePlan {
     std::vector<uint32_t> pubs;
     std::vector<TileLink> links;
 };
+// Orders a tile table: most links first, those without boundary rules last.
+void tile_sort(std::vector<TileRec> &tiles);
+// A launch with so many interior tiles per SM is two kernels.  Us per launch in
+// two kernels and in one: 800^2 (1.2 tiles per SM) 48.7 and 42.3, 1000^2 (2.1)
+// 55.0 and 55.2, 1300^2 (4.1) 81.6 and 83.3, 2048^2 (11) 183.2 and 186.3; with
+// lambda != mu 800^2 (2.0) 34.8 and 35.2, 1000^2 45.6 and 48.6, 2048^2 170.5 and
+// 184.6.
+constexpr int kSplitTiles = 2;
+// Tiles of an ordered table that take a kernel of their own in a launch of two.
+int tile_rules(const TilePlan &plan, int sms);
 // Cuts the lattice into tiles of a shape; false if a tile would have to
 // publish more nodes than its shape holds (never with shape 0).
 bool tile_plan(const Tables &t, bool wall_node, int shape, TilePlan *p);
@@ -304,6 +314,8 @@ void tile_choose(const Tables &t, bool grad, bool wall_node, int sms, TilePlan *
 struct TileDev {
     CUtensorMap map[2];  // the population buffers, box of one tile
     int shape = -1, ntiles = 0, sms = 1;
+    // where a launch is two kernels, the first of tiles [0, nrules); 0: one kernel
+    int nrules = 0;
     const TileRec *tiles = nullptr;
     const uint32_t *pubs = nullptr;
     const TileLink *links = nullptr;
@@ -323,7 +335,7 @@ struct TileInst {
     Lattice L;
 };
 struct TileBatch {
-    int shape = -1, ntiles = 0, sms = 1;
+    int shape = -1, ntiles = 0, nrules = 0, sms = 1;  // as in TileDev
     bool force = false;  // some instance has a body force
     const TileInst *insts = nullptr;
     const TileRec *tiles = nullptr;

@@ -365,6 +365,14 @@ template <class Use> void for_rings(const BNode &b, int W, int H, int ntx, int n
 
 }  // namespace
 
+// Tiles with links first: they take longest.  Those without come last, the
+// ones with nothing to publish behind the others.
+void tile_sort(std::vector<TileRec> &tiles) {
+    std::stable_sort(tiles.begin(), tiles.end(), [](const TileRec &a, const TileRec &b) {
+        return a.nlink != b.nlink ? a.nlink > b.nlink : a.npub > b.npub;
+    });
+}
+
 bool tile_plan(const Tables &t, bool wall_node, int shape, TilePlan *p) {
     const TileShape sh = kTileShapes[shape];
     const int W = sh.w(), H = sh.h(), sx = W - 2 * kTileHalo, sy = H - 2 * kTileHalo;
@@ -460,15 +468,16 @@ bool tile_plan(const Tables &t, bool wall_node, int shape, TilePlan *p) {
             r.nlink = (uint16_t)(p->links.size() - r.link0);
             p->tiles.push_back(r);
         }
-    // tiles with links first: they take longest
-    std::stable_sort(p->tiles.begin(), p->tiles.end(),
-                     [](const TileRec &a, const TileRec &b) { return a.nlink > b.nlink; });
+    tile_sort(p->tiles);
     return true;
 }
 
-namespace {
-
-}  // namespace
+int tile_rules(const TilePlan &plan, int sms) {
+    if (kTileShapes[plan.shape].rows < 3) return 0;
+    int n = 0;
+    while (n < (int)plan.tiles.size() && plan.tiles[(size_t)n].npub) ++n;
+    return (int)plan.tiles.size() - n >= kSplitTiles * sms ? n : 0;
+}
 
 // Modelled time (us) of one launch with a shape: every tile costs a fixed part
 // (copy in, store) and per step a part for its nodes, one for having boundary

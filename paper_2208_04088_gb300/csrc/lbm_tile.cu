@@ -32,8 +32,8 @@
 // work in 2740).  On lattices of less than a few hundred thousand nodes it is
 // the latency of one step (two block barriers, the collision's and a link's
 // dependent chain: 2 us in a 32 x 32 tile) and of the launch.  2048^2 edge
-// crack, 500 steps: 12.0 ms (strips 18.9); with lambda != mu 24.8 (one step per
-// launch 45.6); 1024 x 512 plate with a hole, 600 steps: 2.55 (4.25).
+// crack, 500 steps: 11.7 ms (strips 18.9); with lambda != mu 21.5 (one step per
+// launch 44.8); 1024 x 512 plate with a hole, 600 steps: 2.52 (4.26).
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
@@ -198,6 +198,7 @@ __device__ __forceinline__ bool load_landed(Control *c, uint32_t bar, uint32_t p
 // nsteps steps of one tile, any tile; the first is step `toff` after *time.
 // `first`: the block's first tile (it waits for the previous launch once its
 // tables are read).  Returns false when the copy did not land in time.
+// late: the next kernel is released only once the previous launch is over.
 // SRC: the source S is not zero (a body force, or the gradient's).
 template <int LPR, int R, bool GRAD, bool SRC>
 __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restrict__ dst,
@@ -208,7 +209,8 @@ __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restr
                                            const BCDev *__restrict__ bcs, const Lattice &L,
                                            const int64_t *__restrict__ time, int toff, int nsteps,
                                            uint32_t *__restrict__ status, unsigned char *sm,
-                                           Control *ctl, bool first, uint32_t load_parity) {
+                                           Control *ctl, bool first, bool late,
+                                           uint32_t load_parity) {
     using S = Shape<LPR, R>;
     constexpr int W = S::W, H = S::H, G = S::G;
     const int tid = threadIdx.x, t = tid % LPR, g = tid / LPR;
@@ -269,6 +271,7 @@ __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restr
     TileLink my_link;
     if (kKeep && tid < nlink) my_link = links[rec.link0 + tid];
     if (first) wait_for_previous();
+    if (late) release_next();
     // while the populations arrive: which of the thread's nodes are material
     // core nodes (bit 2 r + j), and their displacement records
     const float tb0 = (float)(*time + toff - 1);
@@ -751,8 +754,18 @@ __device__ __forceinline__ bool tile_interior(const CUtensorMap *tf, float *__re
         }
         if (tid == 0 && early) take_next(l);
     };
+    if constexpr (GRAD) {  // two at a time: 2048^2 crack 175 us a launch without, 171 with
+        int l = 0;
+        if (!(nsteps & 1)) step(l++, std::false_type{});
 #pragma unroll 1
-    for (int l = 0; l < nsteps - 1; ++l) step(l, std::false_type{});
+        for (; l < nsteps - 1; l += 2) {
+            step(l, std::false_type{});
+            step(l + 1, std::false_type{});
+        }
+    } else {
+#pragma unroll 1
+        for (int l = 0; l < nsteps - 1; ++l) step(l, std::false_type{});
+    }
     step(nsteps - 1, std::true_type{});
     if (!isfinite(nonfinite)) flag_nonfinite(status, nonfinite, 0.0f, 0.0f);
     return true;
@@ -806,10 +819,26 @@ struct BatchLattices {
     __device__ uint32_t *status(int i) const { return insts[i].status; }
 };
 
-// The tiles of a launch.  Tiles of 64 columns are taken by one block per SM,
-// the first by block index and the others from a counter, which the last block
-// to finish puts back to zero; the smallest tiles go one to a block.
-template <int LPR, int R, bool GRAD, bool SRC, class Ctx>
+// A launch is one kernel over all its tiles, or, where it has many without
+// boundary rules (kSplitTiles), two: the first steps the tiles with rules, the
+// second the others.  Each then has registers and code of its own: in the one
+// kernel the interior tiles of the 2048^2 crack take 151 us a launch, alone 145,
+// with lambda != mu 169 and 147.  But the second starts only when the launch
+// before is over, where the one kernel has its blocks waiting.
+//
+// Order of the two: both read what the launch before wrote, and write disjoint
+// cores.  A block of the first waits for the launch before and only then
+// releases the second kernel, whose blocks so find everything they read in
+// place; they start as the first kernel's blocks leave room, and wait for that
+// kernel before they exit: whatever follows the second follows both.
+// The plans with so many tiles take the larger shapes.
+constexpr bool can_split(int lpr, int r) { return lpr == 32 && r >= 3; }
+enum class Part { kAll, kRules, kInner };
+
+// Tiles of 64 columns are taken by one block per SM, the first by block index
+// and the others from a counter, which the last block to finish puts back to
+// zero; the smallest tiles and those of Part::kRules go one to a block.
+template <int LPR, int R, bool GRAD, bool SRC, Part P, class Ctx>
 __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ tiles, int ntiles,
                                           int32_t *__restrict__ counter,
                                           const uint32_t *__restrict__ pubs,
@@ -817,7 +846,7 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
                                           unsigned char *sm) {
     constexpr size_t kControl = control_at<LPR, R, GRAD>();
     Control *ctl = reinterpret_cast<Control *>(sm + kControl);
-    release_next();
+    if (P != Part::kRules) release_next();
     if (threadIdx.x == 0) {
         mbar_init(smem_addr(&ctl->load), 1);
         mbar_init(smem_addr(&ctl->step), kNT / 32);
@@ -827,10 +856,10 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
     __syncthreads();
     TileRec rec = tiles[blockIdx.x];
     ctx.enter(rec.inst);
-    if constexpr (LPR != 32) {
+    if constexpr (LPR != 32 || P == Part::kRules) {
         tile_steps<LPR, R, GRAD, SRC>(ctx.map(rec.inst), ctx.dst(rec.inst), ctx.uc(rec.inst), ctx.cls(rec.inst),
                                  rec, pubs, links, ctx.bcs(rec.inst), ctx.L(), ctx.time(rec.inst), toff,
-                                 nsteps, ctx.status(rec.inst), sm, ctl, true, 0);
+                                 nsteps, ctx.status(rec.inst), sm, ctl, true, P == Part::kRules, 0);
     } else {
         const bool more = ntiles > (int)gridDim.x;
         auto grab = [&]() {
@@ -852,20 +881,20 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
         };
         // whether the next tile is known to every thread before this one's last step
         const bool early = nsteps >= (GRAD ? 4 : 5);
-        bool first = true, loaded = false;
+        bool first = P == Part::kAll, loaded = false;
         uint32_t parity = 0, phase = 0, dphase = 0;
         for (;;) {
             bool ok;
             const int i = rec.inst;
-            const bool ahead = rec.npub == 0 && early;
-            if (rec.npub == 0) {
+            const bool ahead = (P == Part::kInner || rec.npub == 0) && early;
+            if (P == Part::kInner || rec.npub == 0) {
                 ok = tile_interior<R, GRAD, SRC>(ctx.map(i), ctx.dst(i), ctx.uc(i), rec, ctx.L(), nsteps,
                                             ctx.status(i), sm, ctl, first, loaded, early, parity, phase,
                                             dphase, take_next);
             } else {
                 ok = tile_steps<LPR, R, GRAD, SRC>(ctx.map(i), ctx.dst(i), ctx.uc(i), ctx.cls(i), rec, pubs,
                                               links, ctx.bcs(i), ctx.L(), ctx.time(i), toff, nsteps,
-                                              ctx.status(i), sm, ctl, first, parity);
+                                              ctx.status(i), sm, ctl, first, false, parity);
             }
             if (!ok) break;  // uniform
             first = false;
@@ -888,10 +917,11 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
             counter[0] = 0;
             counter[1] = 0;
         }
+        if (P == Part::kInner) wait_for_previous();
     }
 }
 
-template <int LPR, int R, bool GRAD, bool SRC>
+template <int LPR, int R, bool GRAD, bool SRC, Part P>
 __global__ void __launch_bounds__(kNT, 1)
     k_tile(const __grid_constant__ CUtensorMap tf, float *__restrict__ dst, float4 *__restrict__ uc,
            const uint8_t *__restrict__ cls, const TileRec *__restrict__ tiles, int ntiles,
@@ -900,29 +930,29 @@ __global__ void __launch_bounds__(kNT, 1)
            const __grid_constant__ Lattice L, const int64_t *__restrict__ time, int toff, int nsteps,
            uint32_t *__restrict__ status) {
     extern __shared__ __align__(1024) unsigned char sm[];
-    run_tiles<LPR, R, GRAD, SRC>(OneLattice{&tf, dst, uc, cls, bcs, L, time, status}, tiles, ntiles, counter,
-                            pubs, links, toff, nsteps, sm);
+    run_tiles<LPR, R, GRAD, SRC, P>(OneLattice{&tf, dst, uc, cls, bcs, L, time, status}, tiles, ntiles,
+                                    counter, pubs, links, toff, nsteps, sm);
 }
 
 // The tiles of many lattices in one launch (a batch, lambda = mu).
-template <int LPR, int R, bool SRC>
+template <int LPR, int R, bool SRC, Part P>
 __global__ void __launch_bounds__(kNT, 1)
     k_tile_batch(const TileInst *__restrict__ insts, const TileRec *__restrict__ tiles, int ntiles,
                  int32_t *__restrict__ counter, const uint32_t *__restrict__ pubs,
                  const TileLink *__restrict__ links, int cur, int toff, int nsteps) {
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(16) Lattice s_L;
-    run_tiles<LPR, R, false, SRC>(BatchLattices{insts, cur, &s_L, -1}, tiles, ntiles, counter, pubs, links,
-                             toff, nsteps, sm);
+    run_tiles<LPR, R, false, SRC, P>(BatchLattices{insts, cur, &s_L, -1}, tiles, ntiles, counter, pubs, links,
+                                     toff, nsteps, sm);
 }
 
-// One launch of `kernel` over a plan's tiles, in programmatic order.
-template <int LPR, int R, bool GRAD, class... P, class... A>
-cudaError_t launch_tiles(void (*kernel)(P...), int ntiles, int sms, cudaStream_t s, A... args) {
+// `kernel` in programmatic order behind the one launched before it.
+template <class... P, class... A>
+cudaError_t launch_tiles(void (*kernel)(P...), int blocks, size_t smem, cudaStream_t s, A... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(LPR == 32 ? std::min(ntiles, sms) : ntiles));
+    cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(kNT);
-    cfg.dynamicSmemBytes = smem_bytes<LPR, R, GRAD>();
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -932,24 +962,59 @@ cudaError_t launch_tiles(void (*kernel)(P...), int ntiles, int sms, cudaStream_t
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// blocks for n tiles of one launch: one per SM, the smallest tiles one each
+template <int LPR> int blocks_for(int n, int sms) { return LPR == 32 ? std::min(n, sms) : n; }
+
 template <int LPR, int R, bool SRC>
 cudaError_t batch_shape(const TileBatch &B, int cur, int toff, int nsteps, cudaStream_t s) {
-    static const cudaError_t attr_set =
-        cudaFuncSetAttribute(k_tile_batch<LPR, R, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_bytes<LPR, R, false>());
+    auto allow = [](auto kernel) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem_bytes<LPR, R, false>());
+    };
+    static const cudaError_t attr_set = [&] {
+        cudaError_t e = allow(k_tile_batch<LPR, R, SRC, Part::kAll>);
+        if constexpr (can_split(LPR, R)) {
+            if (e == cudaSuccess) e = allow(k_tile_batch<LPR, R, SRC, Part::kRules>);
+            if (e == cudaSuccess) e = allow(k_tile_batch<LPR, R, SRC, Part::kInner>);
+        }
+        return e;
+    }();
     if (attr_set != cudaSuccess || B.ntiles <= 0) return attr_set;
-    return launch_tiles<LPR, R, false>(k_tile_batch<LPR, R, SRC>, B.ntiles, B.sms, s, B.insts, B.tiles,
-                                       B.ntiles, B.counter, B.pubs, B.links, cur, toff, nsteps);
+    auto launch = [&](auto kernel, int blocks, int first, int n) {
+        return launch_tiles(kernel, blocks, smem_bytes<LPR, R, false>(), s, B.insts, B.tiles + first, n,
+                            B.counter, B.pubs, B.links, cur, toff, nsteps);
+    };
+    if constexpr (can_split(LPR, R)) {
+        if (B.nrules > 0) {
+            const int inner = B.ntiles - B.nrules;
+            const cudaError_t e =
+                launch(k_tile_batch<LPR, R, SRC, Part::kRules>, B.nrules, 0, B.nrules);
+            return e != cudaSuccess ? e : launch(k_tile_batch<LPR, R, SRC, Part::kInner>,
+                                                 blocks_for<LPR>(inner, B.sms), B.nrules, inner);
+        }
+    }
+    return launch(k_tile_batch<LPR, R, SRC, Part::kAll>, blocks_for<LPR>(B.ntiles, B.sms), 0, B.ntiles);
 }
 
 template <int LPR, int R, bool GRAD, bool SRC>
 cudaError_t launch_shape(const Lattice &L, const DevState &S, const TileDev &T, int cur, int toff,
                          int nsteps, cudaStream_t s) {
-    return launch_tiles<LPR, R, GRAD>(k_tile<LPR, R, GRAD, SRC>, T.ntiles, T.sms, s, T.map[cur],
-                                      static_cast<float *>(S.f[cur ^ 1]), static_cast<float4 *>(S.ucomp),
-                                      (const uint8_t *)S.cls, T.tiles, T.ntiles, T.counter, T.pubs, T.links,
-                                      (const BCDev *)S.bcs, L, (const int64_t *)S.time, toff, nsteps,
-                                      S.status);
+    auto launch = [&](auto kernel, int blocks, int first, int n) {
+        return launch_tiles(kernel, blocks, smem_bytes<LPR, R, GRAD>(), s, T.map[cur],
+                            static_cast<float *>(S.f[cur ^ 1]), static_cast<float4 *>(S.ucomp),
+                            (const uint8_t *)S.cls, T.tiles + first, n, T.counter, T.pubs, T.links,
+                            (const BCDev *)S.bcs, L, (const int64_t *)S.time, toff, nsteps, S.status);
+    };
+    if constexpr (can_split(LPR, R)) {
+        if (T.nrules > 0) {
+            const int inner = T.ntiles - T.nrules;
+            const cudaError_t e =
+                launch(k_tile<LPR, R, GRAD, SRC, Part::kRules>, T.nrules, 0, T.nrules);
+            return e != cudaSuccess ? e : launch(k_tile<LPR, R, GRAD, SRC, Part::kInner>,
+                                                 blocks_for<LPR>(inner, T.sms), T.nrules, inner);
+        }
+    }
+    return launch(k_tile<LPR, R, GRAD, SRC, Part::kAll>, blocks_for<LPR>(T.ntiles, T.sms), 0, T.ntiles);
 }
 
 template <int LPR, int R>
@@ -965,16 +1030,25 @@ bool encode_shape(const Lattice &L, const DevState &S, CUtensorMap map[2]) {
 
 bool has_force(const Lattice &L) { return L.fx != 0.0f || L.fy != 0.0f; }
 
+template <int LPR, int R, bool GRAD, bool SRC> cudaError_t allow_smem() {
+    auto allow = [](auto kernel) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem_bytes<LPR, R, GRAD>());
+    };
+    cudaError_t e = allow(k_tile<LPR, R, GRAD, SRC, Part::kAll>);
+    if constexpr (can_split(LPR, R)) {
+        if (e == cudaSuccess) e = allow(k_tile<LPR, R, GRAD, SRC, Part::kRules>);
+        if (e == cudaSuccess) e = allow(k_tile<LPR, R, GRAD, SRC, Part::kInner>);
+    }
+    return e;
+}
+
 template <int LPR, int R> cudaError_t prepare_shape(const Lattice &L, const DevState &S, TileDev *T) {
     if (!encode_shape<LPR, R>(L, S, T->map)) return cudaErrorInvalidValue;
-    auto limit = [](auto kernel, size_t bytes) {
-        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    };
     if constexpr (R < 4)
-        if (L.grad) return limit(k_tile<LPR, R, true, true>, smem_bytes<LPR, R, true>());
+        if (L.grad) return allow_smem<LPR, R, true, true>();
     if (L.grad) return cudaErrorInvalidValue;
-    return has_force(L) ? limit(k_tile<LPR, R, false, true>, smem_bytes<LPR, R, false>())
-                        : limit(k_tile<LPR, R, false, false>, smem_bytes<LPR, R, false>());
+    return has_force(L) ? allow_smem<LPR, R, false, true>() : allow_smem<LPR, R, false, false>();
 }
 
 }  // namespace
