@@ -37,17 +37,19 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "GLUPS (giga lattice updates per second, whole job)"
-# FP32 operations of one lattice update in the temporally blocked kernel (FMA =
-# 2): raw moments 24, relaxation 26, populations 30, displacement update 11
-FLOPS_PER_UPDATE = 91
-# with lambda != mu the blocked kernel also forms each node's density (8) and
-# the source from the density gradient (10)
-FLOPS_PER_UPDATE_GRAD = 109
+# FP32 operations of one lattice update in the temporally blocked kernels (FMA =
+# 2): moments and populations 39, 13 of them FMAs, displacement update 11
+FLOPS_PER_UPDATE = 63
+# with lambda != mu also the source from the density gradient (10) and its eight
+# FMAs in the collision
+FLOPS_PER_UPDATE_GRAD = 89
 # the kernel sources each kernel's recorded DRAM traffic depends on
 KERNEL_SOURCES = {"k_interior": ("lbm_kernels.cu", "lbm_device.cuh"),
                   "k_interior_pair": ("lbm_kernels.cu", "lbm_device.cuh", "lbm_pair.cuh"),
                   "k_interior_grad": ("lbm_kernels.cu", "lbm_device.cuh"),
                   "k_interior_aa": ("lbm_kernels.cu", "lbm_device.cuh"),
+                  "k_tile": ("lbm_tile.cu", "lbm_async.cuh", "lbm_device.cuh"),
+                  "k_tile_grad": ("lbm_tile.cu", "lbm_async.cuh", "lbm_device.cuh"),
                   "k_wave": ("lbm_wave.cu", "lbm_device.cuh"),
                   "k_wave_grad": ("lbm_wave.cu", "lbm_device.cuh")}
 WORKLOADS = ("crack", "plate", "batch", "serve")
@@ -255,6 +257,12 @@ def _alu_peak_tflops(dev, sm_mhz):
     return sms * 128 * 2 * sm_mhz * 1e6 / 1e12, sms
 
 
+def _blocked_kernel(time_block, lam_over_mu):
+    """Name of the temporally blocked kernel: the register tiles by default (with
+    lambda != mu their other form), the strips on request."""
+    return ("k_wave" if time_block else "k_tile") + ("" if lam_over_mu == 1.0 else "_grad")
+
+
 def _roofline_blocked(nodes, tblock, mean_launch_ms, bytes_per_update, lam_over_mu, hbm_peak,
                       hbm_kind, clk, dev):
     """Roofline of one temporally blocked launch: the HBM ceiling (one pass of
@@ -350,7 +358,7 @@ def _variant_record(wl, args, dev, stream, storage, wall_node, time_block, solve
         clk = {"sm_mhz": None}  # the nominal maximum clock for this secondary record
         roof = _roofline_blocked(nodes, tb, mean_ms, info["bytes_per_update"], wl.lam_over_mu,
                                  peak, peak_kind, clk, dev)
-        roof["kernel"] = "k_wave" if wl.lam_over_mu == 1.0 else "k_wave_grad"
+        roof["kernel"] = _blocked_kernel(time_block, wl.lam_over_mu)
     else:
         mean_ms = tim["interior_ms"] / max(1, tim["steps"])
         gbs = info["interior_nodes"] * info["bytes_per_update"] / (mean_ms * 1e-3) / 1e9
@@ -802,7 +810,7 @@ def run_gpu(args):
         # allows the smaller throughput, i.e. the longer minimum launch time.
         n_launch = max(1, tim["steps"] // tblock)
         mean_launch_ms = tim["interior_ms"] / n_launch
-        kname = "k_wave" if wl.lam_over_mu == 1.0 else "k_wave_grad"
+        kname = _blocked_kernel(args.time_block, wl.lam_over_mu)
         roofline = _roofline_blocked(nodes, tblock, mean_launch_ms, info0["bytes_per_update"],
                                      wl.lam_over_mu, peak, peak_kind, clk, dev)
         roofline.update({

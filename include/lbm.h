@@ -226,7 +226,7 @@ lbm_status lbm_workspace_size(const lbm_desc *desc, uint64_t *bytes);
  * lbm_workspace_size() bytes, 256-byte aligned, owned by the caller and kept
  * alive until lbm_destroy; otherwise the library allocates with cudaMalloc.
  * The caller keeps ownership of every host array; none is referenced after
- * return.  With temporal blocking, three blocked launches on the zero state
+ * return.  With blocking in strips, three blocked launches on the zero state
  * measure the SM cycles of every block and the strips are re-cut to balance
  * them (a launch plan with the smallest measured maximum is kept; a lattice
  * created again in the same process reuses it); the state is then reset.
@@ -286,17 +286,19 @@ lbm_status lbm_sync(lbm_handle h);
 lbm_status lbm_get_info(lbm_handle h, lbm_info *info);
 
 /* Limit of every bounded wait inside the kernels (the temporally blocked
- * kernels wait for the tile copies of their input rows), in nanoseconds;
+ * kernels wait for the copies of their input), in nanoseconds;
  * 0 .. 60e9, default 1e9 (1 s).  The paper has no counterpart; this is a
  * service of the library.  After a wait runs out the block issues no further
- * copy and finishes its sweep on whatever its shared-memory rows hold (every
+ * copy.  A block of register tiles then exits without storing the tile; a block
+ * of strips finishes its sweep on whatever its shared-memory rows hold (every
  * table index it reads from them is clamped into its table, so all accesses
- * stay in bounds); it then waits for every copy it still has in flight, each
- * with the default limit, and exits.  lbm_sync and the next lbm_step return
- * then undefined until lbm_reset.  A limit of 0 makes every block give up at
- * its first wait, whether or not that copy has landed, so every blocked launch
- * reports LBM_ERR_TIMEOUT: it exists to test this path.  Synchronises the handle's stream; takes effect
- * from the next step.  LBM_ERR_ARG for a NULL handle or a limit out of range. */
+ * stay in bounds).  Either waits for every copy it still has in flight, each
+ * with the default limit, before it exits.  lbm_sync and the next lbm_step
+ * return LBM_ERR_TIMEOUT; the fields are then undefined until lbm_reset.  A
+ * limit of 0 makes every block give up at its first wait, whether or not that
+ * copy has landed, so every blocked launch reports LBM_ERR_TIMEOUT: it exists
+ * to test this path.  Synchronises the handle's stream; takes effect from the
+ * next step.  LBM_ERR_ARG for a NULL handle or a limit out of range. */
 lbm_status lbm_set_wait_limit(lbm_handle h, int64_t limit_ns);
 
 /* Timing mode for profiling.  While enabled, lbm_step launches the kernels of

@@ -409,10 +409,10 @@ lbm_status create_prepared(const lbm_desc *desc, Tables &&tab, const Units &unit
                             cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = launch_reset(h->storage, h->L, S, h->stream);
     // The default takes register tiles wherever their modelled time is below
-    // one step per launch: 8 steps of a 64^2 plate in 17 us against 35, of a
-    // 1024 x 512 plate in 34 against 57, of the 2048^2 crack in 192 us against
+    // one step per launch: 8 steps of a 64^2 plate in 15 us against 35, of a
+    // 1024 x 512 plate in 34 against 57, of the 2048^2 crack in 183 us against
     // 300 in strips (k_wave, 538 one step at a time), and with lambda != mu 4
-    // steps of the crack in 198 us against 364 (strips: 349).
+    // steps of the crack in 171 us against 359 (strips: 349).
     if (e == cudaSuccess && desc->time_block == 0 &&
         h->storage == LBM_F32 && !in_place)
         e = tile_create(h);

@@ -543,8 +543,8 @@ void tile_choose(const Tables &t, bool grad, bool wall_node, int sms, TilePlan *
     // from the largest tile down; once a shape fills the SMs several times
     // over, smaller tiles only add halo
     // (with lambda != mu the densities leave too few registers for four rows to
-    // a thread: 2048^2 in 64 x 64 tiles 121 us a launch of 4 steps, in 64 x 48
-    // 103)
+    // a thread: the interior tiles of 2048^2 take 191 us a launch of 4 steps in
+    // 64 x 64 tiles, 147 in 64 x 48)
     for (int s = kTileShapeCount - (grad ? 2 : 1); s >= 0; --s) {
         order.emplace_back(tile_time(t, s, grad, sms), s);
         if ((size_t)ring_count(t.nx, kTileShapes[s].w()) * ring_count(t.ny, kTileShapes[s].h()) >
