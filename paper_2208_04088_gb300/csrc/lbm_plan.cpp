@@ -480,15 +480,18 @@ int tile_rules(const TilePlan &plan, int sms) {
 }
 
 // Modelled time (us) of one launch with a shape: every tile costs a fixed part
-// (copy in, store) and per step a part for its nodes, one for having boundary
-// rules at all (two more barriers and a link's dependent chain) and one per
-// link; the tiles, those with links first, are taken by `sms` SMs, one each.
-// Constants per shape from GB300 timings of lattices of 64^2 to 2048^2 nodes (8 steps: 17 us for a
-// wave of 32 x 32 tiles with links, 9 us without; 24 us for 64 x 64 without).
+// (copy in, store; tiles without rules copy the next one in meanwhile) and per
+// step a part for its nodes, one for having boundary rules at all (two more
+// barriers and a link's dependent chain) and one per link; the tiles, those
+// with links first, are taken by `sms` SMs, one each.  Constants per shape from
+// GB300 timings of plates and cracks of 64^2 to 2048^2 nodes (8 steps: 14, 20.5,
+// 26 and 31.5 us for one wave of tiles with links, 14 for an interior tile of
+// 64 x 64).
 double tile_time(const Tables &t, int shape, bool grad, int sms) {
-    static const double kFixed[kTileShapeCount] = {4.0, 5.0, 6.0, 6.5};
-    static const double kNodes[kTileShapeCount] = {0.7, 1.2, 1.6, 1.75};
-    static const double kRules[kTileShapeCount] = {0.7, 1.3, 1.6, 1.9};
+    static const double kFixed[kTileShapeCount] = {4.0, 4.5, 5.0, 5.5};
+    static const double kInner[kTileShapeCount] = {1.4, 2.0, 2.0, 2.0};
+    static const double kNodes[kTileShapeCount] = {0.5, 0.75, 1.1, 1.5};
+    static const double kRules[kTileShapeCount] = {0.7, 1.2, 1.5, 1.75};
     const double kLink = 0.0008;
     const int W = kTileShapes[shape].w(), H = kTileShapes[shape].h();
     const int ntx = ring_count(t.nx, W), nty = ring_count(t.ny, H);
@@ -498,7 +501,8 @@ double tile_time(const Tables &t, int shape, bool grad, int sms) {
         const int n = __builtin_popcount(b.cut);
         for_rings(b, W, H, ntx, nty, [&](size_t k) { links[k] += n; });
     }
-    const double plain = kFixed[shape] + steps * (grad ? 1.3 : 1.0) * kNodes[shape];
+    const double nodes = steps * (grad ? 1.3 : 1.0) * kNodes[shape];
+    const double plain = kInner[shape] + nodes;
     // the tiles with links go first, in order; the others fill up evenly
     std::priority_queue<double, std::vector<double>, std::greater<double>> sm;
     for (int k = 0; k < sms; ++k) sm.push(0.0);
@@ -509,7 +513,7 @@ double tile_time(const Tables &t, int shape, bool grad, int sms) {
             ++without;
             continue;
         }
-        const double c = plain + steps * ((grad ? 1.5 : 1.0) * kRules[shape] + kLink * n);
+        const double c = kFixed[shape] + nodes + steps * ((grad ? 1.5 : 1.0) * kRules[shape] + kLink * n);
         const double at = sm.top() + c;
         sm.pop();
         sm.push(at);
