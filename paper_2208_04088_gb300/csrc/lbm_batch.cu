@@ -149,11 +149,11 @@ __global__ void __launch_bounds__(TX *TY, kBatchThreadsPerSm<T, kMixed> / (TX * 
                 if (kMixed && I.L.in_place) {  // one buffer: the AA step of the instance's parity
                     T *f = static_cast<T *>(I.f[0]);
                     if (cur)
-                        interior_node<T, kAAOdd>(f, f, static_cast<URec<T> *>(I.uc), I.cls, nullptr, I.L, k, I.status);
+                        interior_node<T, kAAOdd, true>(f, f, static_cast<URec<T> *>(I.uc), I.cls, nullptr, I.L, k, I.status);
                     else
-                        interior_node<T, kAAEven>(f, f, static_cast<URec<T> *>(I.uc), I.cls, nullptr, I.L, k, I.status);
+                        interior_node<T, kAAEven, true>(f, f, static_cast<URec<T> *>(I.uc), I.cls, nullptr, I.L, k, I.status);
                 } else {
-                    interior_node<T>(static_cast<const T *>(I.f[cur]),
+                    interior_node<T, kPull, true>(static_cast<const T *>(I.f[cur]),
                                      static_cast<T *>(I.f[cur ^ 1]), static_cast<URec<T> *>(I.uc), I.cls, nullptr, I.L, k,
                                      I.status);
                 }

@@ -988,9 +988,11 @@ __device__ __forceinline__ void source_boundary8(const T *__restrict__ src,
 // One interior node: pull (Eq. stream), moments with the source, collision
 // (Eq. coll), store, displacement.  Every load -- the nine pulled
 // populations and the displacement record -- is issued before any arithmetic.
+// kBatch: lambda = mu, and the record is loaded behind the stores, which keeps
+// the batched kernel within its 32 registers without spills.
 // With kAA src and dst are the same buffer: the node reads all nine of its
 // locations before it writes any.
-template <class T, int LAY = kPull>
+template <class T, int LAY = kPull, bool kBatch = false>
 __device__ __forceinline__ void interior_node(const T *src, T *dst, URec<T> *__restrict__ uc,
                                               const uint8_t *__restrict__ cls,
                                               const float *__restrict__ rho, const Lattice &L,
@@ -998,13 +1000,18 @@ __device__ __forceinline__ void interior_node(const T *src, T *dst, URec<T> *__r
     if (__ldg(cls + k) != kInterior) return;
     float f[9];
     pull_interior_at<LAY>(src, k, L, f);
-    URec<T> w = uc[k];
+    URec<T> w;
+    if (!kBatch) w = uc[k];
     float sx = L.fx, sy = L.fy;
-    if (L.grad) source_interior(rho, k, L.pitch, rho[k], L, sx, sy);
+    if (!kBatch && L.grad) source_interior(rho, k, L.pitch, rho[k], L, sx, sy);
     float dr, jx, jy;
     collide<kSumsOf<T>>(f, sx, sy, L, dr, jx, jy);
 #pragma unroll
     for (int i = 0; i < 9; ++i) Store<T>::st(dst + out_at<LAY>(k, i, L), f[i], L.scale);
+    if (kBatch) {
+        asm volatile("" ::: "memory");  // not hoisted above the stores
+        w = uc[k];
+    }
     if constexpr (std::is_same<T, __half>::value) {
         float m = 0.0f;
 #pragma unroll
