@@ -363,6 +363,14 @@ template <class Use> void for_rings(const BNode &b, int W, int H, int ntx, int n
         for (int tx = tx1; tx >= 0 && b.x < tx * sx + W; --tx) use((size_t)ty * ntx + tx);
 }
 
+// Whether ring (tx, ty), which holds the node, ever computes it: its outermost
+// nodes beside a neighbouring ring it does not.
+bool computed(const BNode &b, int tx, int ty, int W, int H, int ntx, int nty) {
+    const int c = b.x - tx * (W - 2 * kTileHalo), row = b.y - ty * (H - 2 * kTileHalo);
+    return (tx == 0 || c >= 1) && (tx == ntx - 1 || c <= W - 2) && (ty == 0 || row >= 1) &&
+           (ty == nty - 1 || row <= H - 2);
+}
+
 }  // namespace
 
 // Tiles with links first: they take longest.  Those without come last, the
@@ -422,11 +430,7 @@ bool tile_plan(const Tables &t, bool wall_node, int shape, TilePlan *p) {
                 const int32_t gi = seen[(size_t)q];
                 const BNode &b = t.bnodes[gi];
                 const int c = b.x - r.x0, row = b.y - r.y0;
-                // the ring's outermost nodes beside a neighbouring tile are
-                // never computed
-                if ((tx > 0 && c < 1) || (tx < ntx - 1 && c > W - 2) || (ty > 0 && row < 1) ||
-                    (ty < nty - 1 && row > H - 2))
-                    continue;
+                if (!computed(b, tx, ty, W, H, ntx, nty)) continue;
                 const int own = publish(c, row);
                 p->pubs[r.pub0 + own] |= (uint32_t)((b.cut >> 1) & 0xffu) << 16;
                 for (int i = 1; i < kQ; ++i) {
@@ -499,7 +503,9 @@ double tile_time(const Tables &t, int shape, bool grad, int sms) {
     std::vector<int32_t> links((size_t)ntx * nty, 0);
     for (const BNode &b : t.bnodes) {
         const int n = __builtin_popcount(b.cut);
-        for_rings(b, W, H, ntx, nty, [&](size_t k) { links[k] += n; });
+        for_rings(b, W, H, ntx, nty, [&](size_t k) {
+            if (computed(b, (int)(k % ntx), (int)(k / ntx), W, H, ntx, nty)) links[k] += n;
+        });
     }
     const double nodes = steps * (grad ? 1.3 : 1.0) * kNodes[shape];
     const double plain = kInner[shape] + nodes;
