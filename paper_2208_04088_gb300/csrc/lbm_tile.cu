@@ -600,14 +600,7 @@ __device__ __forceinline__ bool tile_interior(const CUtensorMap *tf, float *__re
         copy_wait();
         return false;
     }
-    if (rec.c1 == rec.c0) {  // no material in the whole lattice
-        copy_wait();
-        __syncthreads();
-        if (tid == 0 && early)
-            for (int part = 0; part < 3; ++part) take_next(part);
-        __syncthreads();
-        return true;
-    }
+    if (rec.c1 == rec.c0) return true;  // no material in the whole lattice, nothing copied behind it
     F2 f[R][9];
     {
         // pulled along y by the address (the ring's outermost rows, halo, by
@@ -886,7 +879,8 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
         for (;;) {
             bool ok;
             const int i = rec.inst;
-            const bool ahead = (P == Part::kInner || rec.npub == 0) && early;
+            // an empty core steps nothing, so it takes no tile meanwhile
+            const bool ahead = (P == Part::kInner || rec.npub == 0) && early && rec.c1 > rec.c0;
             if (P == Part::kInner || rec.npub == 0) {
                 ok = tile_interior<R, GRAD, SRC>(ctx.map(i), ctx.dst(i), ctx.uc(i), rec, ctx.L(), nsteps,
                                             ctx.status(i), sm, ctl, first, loaded, early, parity, phase,
