@@ -286,11 +286,14 @@ lbm_status lbm_sync(lbm_handle h);
 lbm_status lbm_get_info(lbm_handle h, lbm_info *info);
 
 /* Limit of every bounded wait inside the kernels (the temporally blocked
- * kernels wait for the copies of their input), in nanoseconds;
+ * kernels wait for the copies of their input, and the warps of a register
+ * tile without boundary nodes for one another's rows), in nanoseconds;
  * 0 .. 60e9, default 1e9 (1 s).  The paper has no counterpart; this is a
- * service of the library.  After a wait runs out the block issues no further
- * copy.  A block of register tiles then exits without storing the tile; a block
- * of strips finishes its sweep on whatever its shared-memory rows hold (every
+ * service of the library.  A block of register tiles whose copy has not landed
+ * in time exits without storing the tile; where a wait between its warps runs
+ * out, no warp that may have been given wrong rows stores any, and the block
+ * takes no further tile.  A block of strips issues no further copy after a wait
+ * that ran out; it finishes its sweep on whatever its shared-memory rows hold (every
  * table index it reads from them is clamped into its table, so all accesses
  * stay in bounds).  Either waits for every copy it still has in flight, each
  * with the default limit, before it exits.  lbm_sync and the next lbm_step

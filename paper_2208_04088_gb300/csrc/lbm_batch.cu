@@ -1037,7 +1037,7 @@ int finish_retired(lbm_engine *E) {
             r.result.assign(R.buf, R.buf + 7 * N);
             r.unstable = (status & 1u) != 0;
             r.state = (status & 2u) ? 3 : 2;
-            if (status & 2u) r.error = "a bounded wait for a tile copy expired on the device";
+            if (status & 2u) r.error = "a bounded wait of a kernel ran out on the device";
         } else {
             r.state = 3;
             r.error = std::string("server: ") + cudaGetErrorString(q);

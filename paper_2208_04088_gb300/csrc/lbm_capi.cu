@@ -461,7 +461,7 @@ extern "C" lbm_status lbm_step(lbm_handle h, int64_t nsteps) {
         if (q == cudaSuccess) {
             h->status_pending = false;
             if (*h->h_status & 2u) {
-                set_error("lbm_step: a bounded wait for a tile copy expired on the device");
+                set_error("lbm_step: a bounded wait of a kernel ran out on the device");
                 return LBM_ERR_TIMEOUT;
             }
             if (*h->h_status & 1u) {
@@ -662,7 +662,7 @@ extern "C" lbm_status lbm_sync(lbm_handle h) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "lbm_sync");
     if (status & 2u) {
-        set_error("lbm_sync: a bounded wait for a tile copy expired on the device");
+        set_error("lbm_sync: a bounded wait of a kernel ran out on the device");
         return LBM_ERR_TIMEOUT;
     }
     if (status & 1u) {

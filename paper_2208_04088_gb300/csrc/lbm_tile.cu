@@ -92,6 +92,7 @@ template <int R, bool GRAD> struct Inner {
 struct Control {
     unsigned long long load, step, den;  // mbarriers: copy landed, rows exchanged, densities exchanged
     int landed, next;                    // the copy landed in time; the block's next tile
+    int lost, pad2;                      // a wait between the block's warps ran out
     TileRec rec;                         // its record
     float4 *uc;                          // and its displacement records
     int pitch, pad;
@@ -181,6 +182,10 @@ __device__ __forceinline__ void issue_load(const CUtensorMap *tf, const TileRec 
 // Block-wide wait for the copy; false after the wait limit: the launch is
 // flagged, and the copy waited out so that none is in flight when the block
 // exits.  A limit of 0 gives up at once, whether or not the copy has landed.
+// Also false where a wait between the block's warps ran out (is_lost).
+__device__ __forceinline__ bool is_lost(const Control *c) {
+    return *reinterpret_cast<const volatile int *>(&c->lost) != 0;
+}
 __device__ __forceinline__ bool load_landed(Control *c, uint32_t bar, uint32_t parity,
                                             const Lattice &L, uint32_t *status) {
     if (threadIdx.x == 0) {
@@ -192,7 +197,7 @@ __device__ __forceinline__ bool load_landed(Control *c, uint32_t bar, uint32_t p
         }
     }
     __syncthreads();
-    return *reinterpret_cast<volatile int *>(&c->landed) != 0;
+    return *reinterpret_cast<volatile int *>(&c->landed) != 0 && !is_lost(c);
 }
 
 // nsteps steps of one tile, any tile; the first is step `toff` after *time.
@@ -562,6 +567,15 @@ __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" 
 // records of its own nodes of the next tile as soon as those of this one are
 // stored.  early: it does (a launch of too few steps takes the next tile
 // afterwards); loaded: the tile before this one did.
+//
+// A wait of the warps for one another that runs out flags the launch and the
+// block (ctl->lost).  The warp goes on, arriving as before, so no later wait is
+// longer than the limit either, but a phase may then end without every warp.  It
+// cannot end so unseen: the flag is stored before the warp's next arrival, which
+// releases it to whoever that arrival lets through.  So a warp that finds the
+// flag clear once its last wait is over has been given everything it used, its
+// own rows and thread 0's words on the next tile; where the flag is set it stores
+// nothing, copies nothing for the next tile, and the block takes no other one.
 template <int R, bool GRAD, bool SRC, class Next>
 __device__ __forceinline__ bool tile_interior(const CUtensorMap *tf, float *__restrict__ dst,
                                               float4 *__restrict__ uc, const TileRec &rec,
@@ -624,6 +638,12 @@ __device__ __forceinline__ bool tile_interior(const CUtensorMap *tf, float *__re
         f[r][6] = from_right<32>(f[r][6]);
         f[r][7] = from_right<32>(f[r][7]);
     };
+    // the end of a phase of a barrier that the block's warps meet at
+    auto meet = [&](uint32_t at, uint32_t parity) {
+        if (mbar_wait(at, parity, L.wait_ns)) return;
+        *reinterpret_cast<volatile int *>(&ctl->lost) = 1;
+        atomicOr(status, 2u);
+    };
     // the outermost rows to the neighbouring warps
     auto post = [&](int l) {
         unsigned long long *eu = ex + (GRAD ? 0 : (l & 1) * I::kExOne) + t, *ed = eu + (G - 1) * 96;
@@ -654,7 +674,7 @@ __device__ __forceinline__ bool tile_interior(const CUtensorMap *tf, float *__re
             f[r][7] = f[r + 1][7];
             f[r][8] = f[r + 1][8];
         }
-        mbar_wait(bstep, phase, kDefaultWaitNs);
+        meet(bstep, phase);
         phase ^= 1;
         const unsigned long long *eu = ex + (GRAD ? 0 : (l & 1) * I::kExOne) + t, *ed = eu + (G - 1) * 96;
         if (g > 0) {
@@ -684,11 +704,12 @@ __device__ __forceinline__ bool tile_interior(const CUtensorMap *tf, float *__re
             if (g > 0) den[(G - 1 + g - 1) * 32 + t] = dn[0].v;
             __syncwarp();
             if (t == 0) mbar_arrive(bden);
-            mbar_wait(bden, dphase, kDefaultWaitNs);
+            meet(bden, dphase);
             dphase ^= 1;
             dbelow = g > 0 ? as_f2(den[(g - 1) * 32 + t]) : dn[0];
             dabove = g < G - 1 ? as_f2(den[(G - 1 + g) * 32 + t]) : dn[R - 1];
         }
+        const bool keep = core && !(last && is_lost(ctl));
         // the thread's two outermost rows first
 #pragma unroll
         for (int q = 0; q < R; ++q) {
@@ -712,7 +733,7 @@ __device__ __forceinline__ bool tile_interior(const CUtensorMap *tf, float *__re
                     float4 wa = *ua, wb = *ub;
                     integrate_u_value(wa, jxa, jya, L.rho0 + dra);
                     integrate_u_value(wb, jxb, jyb, L.rho0 + drb);
-                    if (core) {
+                    if (keep) {
                         if (!last) {
                             *ua = wa;
                             *ub = wb;
@@ -844,6 +865,8 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
         mbar_init(smem_addr(&ctl->load), 1);
         mbar_init(smem_addr(&ctl->step), kNT / 32);
         mbar_init(smem_addr(&ctl->den), kNT / 32);
+        ctl->lost = 0;
+        ctl->next = -1;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -876,6 +899,10 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
         const bool early = nsteps >= (GRAD ? 4 : 5);
         bool first = P == Part::kAll, loaded = false;
         uint32_t parity = 0, phase = 0, dphase = 0;
+        // Where the flag of a wait between warps is set, threads leave as they
+        // see it (a thread that has left counts as arrived at every later
+        // barrier of the block); whoever goes on past a barrier that a thread
+        // has left sees it too, behind that barrier.
         for (;;) {
             bool ok;
             const int i = rec.inst;
@@ -890,10 +917,11 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
                                               links, ctx.bcs(i), ctx.L(), ctx.time(i), toff, nsteps,
                                               ctx.status(i), sm, ctl, first, false, parity);
             }
-            if (!ok) break;  // uniform
+            if (!ok) break;
             first = false;
             parity ^= 1;
             loaded = ahead;
+            if (is_lost(ctl)) break;
             if (!ahead) {
                 if (!more) break;
                 __syncthreads();
@@ -902,10 +930,19 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
                     if (ctl->next >= 0) ctl->rec = tiles[ctl->next];
                 }
                 __syncthreads();
+                if (is_lost(ctl)) break;
             }
             if (ctl->next < 0) break;
             rec = ctl->rec;
             ctx.enter(rec.inst);
+            if (is_lost(ctl)) break;
+        }
+        if (is_lost(ctl)) {
+            // nothing in flight when the block exits: this thread's records, and
+            // thread 0's copy of the next tile
+            copy_wait();
+            if (threadIdx.x == 0 && loaded && ctl->next >= 0)
+                mbar_wait(smem_addr(&ctl->load), parity, kDefaultWaitNs);
         }
         if (more && threadIdx.x == 0 && atomicAdd(counter + 1, 1) == (int)gridDim.x - 1) {
             counter[0] = 0;
