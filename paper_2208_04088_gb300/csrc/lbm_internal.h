@@ -319,7 +319,7 @@ struct TileDev {
     const TileRec *tiles = nullptr;
     const uint32_t *pubs = nullptr;
     const TileLink *links = nullptr;
-    int32_t *counter = nullptr;  // tiles taken, blocks done (both 0 between launches)
+    int32_t *counter = nullptr;  // tiles taken, blocks done and ready (0 between launches)
     void *mem = nullptr;
 };
 // Device record of one instance of a batch stepped in tiles, and the tables of

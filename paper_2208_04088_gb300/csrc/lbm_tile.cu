@@ -160,6 +160,12 @@ __device__ __forceinline__ LinkRule make_rule(const TileLink &lk, const BCDev *_
                      tb, L);
 }
 
+// A wait that did not end at the first try, out of the step's code: 2048^2 crack
+// 11.42 ms, 11.79 with it inline (lambda != mu keeps it inline: 21.7, 23.7).
+__device__ __noinline__ bool wait_on(uint32_t bar, uint32_t parity, int64_t limit) {
+    return mbar_wait(bar, parity, limit);
+}
+
 // Programmatic launch order: the next launch of the stream may start its
 // prologue now, and this one has waited for everything before it.
 __device__ __forceinline__ void release_next() {
@@ -167,6 +173,24 @@ __device__ __forceinline__ void release_next() {
 }
 __device__ __forceinline__ void wait_for_previous() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Between the two kernels of a launch (see Part): a block of the first counts
+// itself in counter[kReady], with what the launch before wrote behind it; the
+// second has all of that once it reads the count of every block.
+constexpr int kReady = 2;
+__device__ __forceinline__ void say_ready(int32_t *counter) {
+    int before;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;"
+                 : "=r"(before)
+                 : "l"(counter + kReady)
+                 : "memory");
+    if (before >= 0) release_next();  // (always) not before the count has arrived
+}
+__device__ __forceinline__ bool all_ready(const int32_t *counter, int blocks) {
+    int n;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(n) : "l"(counter + kReady) : "memory");
+    return n == blocks;
 }
 
 // Copies a tile's populations into the space at the start of shared memory.
@@ -182,10 +206,6 @@ __device__ __forceinline__ void issue_load(const CUtensorMap *tf, const TileRec 
 // Block-wide wait for the copy; false after the wait limit: the launch is
 // flagged, and the copy waited out so that none is in flight when the block
 // exits.  A limit of 0 gives up at once, whether or not the copy has landed.
-// Also false where a wait between the block's warps ran out (is_lost).
-__device__ __forceinline__ bool is_lost(const Control *c) {
-    return *reinterpret_cast<const volatile int *>(&c->lost) != 0;
-}
 __device__ __forceinline__ bool load_landed(Control *c, uint32_t bar, uint32_t parity,
                                             const Lattice &L, uint32_t *status) {
     if (threadIdx.x == 0) {
@@ -197,13 +217,17 @@ __device__ __forceinline__ bool load_landed(Control *c, uint32_t bar, uint32_t p
         }
     }
     __syncthreads();
-    return *reinterpret_cast<volatile int *>(&c->landed) != 0 && !is_lost(c);
+    return *reinterpret_cast<volatile int *>(&c->landed) != 0;
+}
+__device__ __forceinline__ bool is_lost(const Control *c) {
+    return *reinterpret_cast<const volatile int *>(&c->lost) != 0;
 }
 
 // nsteps steps of one tile, any tile; the first is step `toff` after *time.
 // `first`: the block's first tile (it waits for the previous launch once its
 // tables are read).  Returns false when the copy did not land in time.
-// late: the next kernel is released only once the previous launch is over.
+// ready: counter to release the next kernel with (say_ready) once the previous
+// launch is over, or null (released before).
 // SRC: the source S is not zero (a body force, or the gradient's).
 template <int LPR, int R, bool GRAD, bool SRC>
 __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restrict__ dst,
@@ -214,7 +238,7 @@ __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restr
                                            const BCDev *__restrict__ bcs, const Lattice &L,
                                            const int64_t *__restrict__ time, int toff, int nsteps,
                                            uint32_t *__restrict__ status, unsigned char *sm,
-                                           Control *ctl, bool first, bool late,
+                                           Control *ctl, bool first, int32_t *ready,
                                            uint32_t load_parity) {
     using S = Shape<LPR, R>;
     constexpr int W = S::W, H = S::H, G = S::G;
@@ -276,7 +300,7 @@ __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restr
     TileLink my_link;
     if (kKeep && tid < nlink) my_link = links[rec.link0 + tid];
     if (first) wait_for_previous();
-    if (late) release_next();
+    if (ready && tid == 0) say_ready(ready);
     // while the populations arrive: which of the thread's nodes are material
     // core nodes (bit 2 r + j), and their displacement records
     const float tb0 = (float)(*time + toff - 1);
@@ -568,14 +592,15 @@ __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" 
 // stored.  early: it does (a launch of too few steps takes the next tile
 // afterwards); loaded: the tile before this one did.
 //
-// A wait of the warps for one another that runs out flags the launch and the
-// block (ctl->lost).  The warp goes on, arriving as before, so no later wait is
-// longer than the limit either, but a phase may then end without every warp.  It
-// cannot end so unseen: the flag is stored before the warp's next arrival, which
-// releases it to whoever that arrival lets through.  So a warp that finds the
-// flag clear once its last wait is over has been given everything it used, its
-// own rows and thread 0's words on the next tile; where the flag is set it stores
-// nothing, copies nothing for the next tile, and the block takes no other one.
+// A wait of the warps for one another that runs out flags the block (ctl->lost),
+// which flags the launch once the tile is over.  The warp goes on, arriving as
+// before, so no later wait is longer than the limit either, but a phase may then
+// end without every warp.  It cannot end so unseen: the flag is stored before the
+// warp's next arrival, which releases it to whoever that arrival lets through.
+// So a warp that finds the flag clear once its last wait is over has been given
+// everything it used, its neighbours' rows and thread 0's words on the next tile;
+// where the flag is set it stores nothing, copies nothing for the next tile, and
+// the block takes no other one.
 template <int R, bool GRAD, bool SRC, class Next>
 __device__ __forceinline__ bool tile_interior(const CUtensorMap *tf, float *__restrict__ dst,
                                               float4 *__restrict__ uc, const TileRec &rec,
@@ -610,7 +635,7 @@ __device__ __forceinline__ bool tile_interior(const CUtensorMap *tf, float *__re
                 copy16(smem_addr(us + r * I::CW + I::CW / 2), uc + k0 + (int64_t)r * L.pitch + 1);
             }
     }
-    if (!load_landed(ctl, bar, load_parity, L, status)) {
+    if (!load_landed(ctl, bar, load_parity, L, status) || is_lost(ctl)) {
         copy_wait();
         return false;
     }
@@ -640,9 +665,9 @@ __device__ __forceinline__ bool tile_interior(const CUtensorMap *tf, float *__re
     };
     // the end of a phase of a barrier that the block's warps meet at
     auto meet = [&](uint32_t at, uint32_t parity) {
-        if (mbar_wait(at, parity, L.wait_ns)) return;
-        *reinterpret_cast<volatile int *>(&ctl->lost) = 1;
-        atomicOr(status, 2u);
+        if (GRAD ? !mbar_wait(at, parity, L.wait_ns)
+                 : !mbar_try_wait(at, parity) && !wait_on(at, parity, L.wait_ns))
+            *reinterpret_cast<volatile int *>(&ctl->lost) = 1;
     };
     // the outermost rows to the neighbouring warps
     auto post = [&](int l) {
@@ -796,7 +821,7 @@ struct OneLattice {
     const Lattice &l;
     const int64_t *clock;
     uint32_t *flags;
-    __device__ void enter(int) {}
+    __device__ bool enter(int) { return false; }
     __device__ const CUtensorMap *map(int) const { return tf; }
     __device__ float *dst(int) const { return out; }
     __device__ float4 *uc(int) const { return u; }
@@ -812,8 +837,9 @@ struct BatchLattices {
     int cur;
     Lattice *l;  // shared memory
     int staged;
-    __device__ void enter(int i) {
-        if (i == staged) return;  // uniform over the block
+    // whether the block has met at a barrier in it
+    __device__ bool enter(int i) {
+        if (i == staged) return false;  // uniform over the block
         constexpr int kWords = (int)(sizeof(Lattice) / 4);
         __syncthreads();  // the last tile's reads are over
         if (threadIdx.x < kWords)
@@ -821,6 +847,7 @@ struct BatchLattices {
                 reinterpret_cast<const uint32_t *>(&insts[i].L)[threadIdx.x];
         __syncthreads();
         staged = i;
+        return true;
     }
     __device__ const CUtensorMap *map(int i) const { return &insts[i].map[cur]; }
     __device__ float *dst(int i) const { return insts[i].f[cur ^ 1]; }
@@ -841,20 +868,23 @@ struct BatchLattices {
 // before is over, where the one kernel has its blocks waiting.
 //
 // Order of the two: both read what the launch before wrote, and write disjoint
-// cores.  A block of the first waits for the launch before and only then
-// releases the second kernel, whose blocks so find everything they read in
-// place; they start as the first kernel's blocks leave room, and wait for that
-// kernel before they exit: whatever follows the second follows both.
+// cores.  A block of the first waits for the launch before, counts itself ready
+// (a release, which passes on what that wait made visible to it) and only then
+// releases the second kernel, whose blocks start as the first kernel's leave
+// room.  Each of them acquires the count before it reads anything; should it not
+// find all blocks in it, it waits for the first kernel to end.  They also wait
+// for that kernel before they exit: whatever follows the second follows both.
 // The plans with so many tiles take the larger shapes.
 constexpr bool can_split(int lpr, int r) { return lpr == 32 && r >= 3; }
 enum class Part { kAll, kRules, kInner };
 
 // Tiles of 64 columns are taken by one block per SM, the first by block index
 // and the others from a counter, which the last block to finish puts back to
-// zero; the smallest tiles and those of Part::kRules go one to a block.
+// zero; the smallest tiles and those of Part::kRules go one to a block.  nrules:
+// the blocks of the first of two kernels.
 template <int LPR, int R, bool GRAD, bool SRC, Part P, class Ctx>
 __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ tiles, int ntiles,
-                                          int32_t *__restrict__ counter,
+                                          int nrules, int32_t *__restrict__ counter,
                                           const uint32_t *__restrict__ pubs,
                                           const TileLink *__restrict__ links, int toff, int nsteps,
                                           unsigned char *sm) {
@@ -867,6 +897,11 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
         mbar_init(smem_addr(&ctl->den), kNT / 32);
         ctl->lost = 0;
         ctl->next = -1;
+        if (P == Part::kInner) {
+            if (!all_ready(counter, nrules)) wait_for_previous();
+            // and before this thread's copies (asynchronous proxy) read it
+            asm volatile("fence.proxy.async.global;" ::: "memory");
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -875,7 +910,8 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
     if constexpr (LPR != 32 || P == Part::kRules) {
         tile_steps<LPR, R, GRAD, SRC>(ctx.map(rec.inst), ctx.dst(rec.inst), ctx.uc(rec.inst), ctx.cls(rec.inst),
                                  rec, pubs, links, ctx.bcs(rec.inst), ctx.L(), ctx.time(rec.inst), toff,
-                                 nsteps, ctx.status(rec.inst), sm, ctl, true, P == Part::kRules, 0);
+                                 nsteps, ctx.status(rec.inst), sm, ctl, true,
+                                 P == Part::kRules ? counter : nullptr, 0);
     } else {
         const bool more = ntiles > (int)gridDim.x;
         auto grab = [&]() {
@@ -899,29 +935,41 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
         const bool early = nsteps >= (GRAD ? 4 : 5);
         bool first = P == Part::kAll, loaded = false;
         uint32_t parity = 0, phase = 0, dphase = 0;
-        // Where the flag of a wait between warps is set, threads leave as they
-        // see it (a thread that has left counts as arrived at every later
-        // barrier of the block); whoever goes on past a barrier that a thread
-        // has left sees it too, behind that barrier.
+        // Where a wait between the warps ran out, threads leave as they see it (a
+        // thread that has left counts as arrived at every later barrier of the
+        // block); whoever goes on past a barrier that a thread has left sees it
+        // too, behind that barrier.  Nothing is in flight then: neither this
+        // thread's records nor, of thread 0, the copy of the next tile.
+        bool inner;
+        int i;
+        auto leave = [&]() {
+            if (!inner || !is_lost(ctl)) return false;
+            if ((threadIdx.x & 31) == 0) atomicOr(ctx.status(i), 2u);
+            copy_wait();
+            if (threadIdx.x == 0 && loaded && ctl->next >= 0)
+                mbar_wait(smem_addr(&ctl->load), parity, kDefaultWaitNs);
+            return true;
+        };
         for (;;) {
             bool ok;
-            const int i = rec.inst;
+            i = rec.inst;
+            inner = P == Part::kInner || rec.npub == 0;
             // an empty core steps nothing, so it takes no tile meanwhile
-            const bool ahead = (P == Part::kInner || rec.npub == 0) && early && rec.c1 > rec.c0;
-            if (P == Part::kInner || rec.npub == 0) {
+            const bool ahead = inner && early && rec.c1 > rec.c0;
+            if (inner) {
                 ok = tile_interior<R, GRAD, SRC>(ctx.map(i), ctx.dst(i), ctx.uc(i), rec, ctx.L(), nsteps,
                                             ctx.status(i), sm, ctl, first, loaded, early, parity, phase,
                                             dphase, take_next);
             } else {
                 ok = tile_steps<LPR, R, GRAD, SRC>(ctx.map(i), ctx.dst(i), ctx.uc(i), ctx.cls(i), rec, pubs,
                                               links, ctx.bcs(i), ctx.L(), ctx.time(i), toff, nsteps,
-                                              ctx.status(i), sm, ctl, first, false, parity);
+                                              ctx.status(i), sm, ctl, first, nullptr, parity);
             }
             if (!ok) break;
             first = false;
             parity ^= 1;
             loaded = ahead;
-            if (is_lost(ctl)) break;
+            if (leave()) break;
             if (!ahead) {
                 if (!more) break;
                 __syncthreads();
@@ -930,23 +978,16 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
                     if (ctl->next >= 0) ctl->rec = tiles[ctl->next];
                 }
                 __syncthreads();
-                if (is_lost(ctl)) break;
+                if (leave()) break;
             }
             if (ctl->next < 0) break;
             rec = ctl->rec;
-            ctx.enter(rec.inst);
-            if (is_lost(ctl)) break;
-        }
-        if (is_lost(ctl)) {
-            // nothing in flight when the block exits: this thread's records, and
-            // thread 0's copy of the next tile
-            copy_wait();
-            if (threadIdx.x == 0 && loaded && ctl->next >= 0)
-                mbar_wait(smem_addr(&ctl->load), parity, kDefaultWaitNs);
+            if (ctx.enter(rec.inst) && leave()) break;
         }
         if (more && threadIdx.x == 0 && atomicAdd(counter + 1, 1) == (int)gridDim.x - 1) {
             counter[0] = 0;
             counter[1] = 0;
+            counter[kReady] = 0;
         }
         if (P == Part::kInner) wait_for_previous();
     }
@@ -955,25 +996,25 @@ __device__ __forceinline__ void run_tiles(Ctx ctx, const TileRec *__restrict__ t
 template <int LPR, int R, bool GRAD, bool SRC, Part P>
 __global__ void __launch_bounds__(kNT, 1)
     k_tile(const __grid_constant__ CUtensorMap tf, float *__restrict__ dst, float4 *__restrict__ uc,
-           const uint8_t *__restrict__ cls, const TileRec *__restrict__ tiles, int ntiles,
+           const uint8_t *__restrict__ cls, const TileRec *__restrict__ tiles, int ntiles, int nrules,
            int32_t *__restrict__ counter, const uint32_t *__restrict__ pubs,
            const TileLink *__restrict__ links, const BCDev *__restrict__ bcs,
            const __grid_constant__ Lattice L, const int64_t *__restrict__ time, int toff, int nsteps,
            uint32_t *__restrict__ status) {
     extern __shared__ __align__(1024) unsigned char sm[];
     run_tiles<LPR, R, GRAD, SRC, P>(OneLattice{&tf, dst, uc, cls, bcs, L, time, status}, tiles, ntiles,
-                                    counter, pubs, links, toff, nsteps, sm);
+                                    nrules, counter, pubs, links, toff, nsteps, sm);
 }
 
 // The tiles of many lattices in one launch (a batch, lambda = mu).
 template <int LPR, int R, bool SRC, Part P>
 __global__ void __launch_bounds__(kNT, 1)
     k_tile_batch(const TileInst *__restrict__ insts, const TileRec *__restrict__ tiles, int ntiles,
-                 int32_t *__restrict__ counter, const uint32_t *__restrict__ pubs,
+                 int nrules, int32_t *__restrict__ counter, const uint32_t *__restrict__ pubs,
                  const TileLink *__restrict__ links, int cur, int toff, int nsteps) {
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ __align__(16) Lattice s_L;
-    run_tiles<LPR, R, false, SRC, P>(BatchLattices{insts, cur, &s_L, -1}, tiles, ntiles, counter, pubs, links,
+    run_tiles<LPR, R, false, SRC, P>(BatchLattices{insts, cur, &s_L, -1}, tiles, ntiles, nrules, counter, pubs, links,
                                      toff, nsteps, sm);
 }
 
@@ -1013,7 +1054,7 @@ cudaError_t batch_shape(const TileBatch &B, int cur, int toff, int nsteps, cudaS
     if (attr_set != cudaSuccess || B.ntiles <= 0) return attr_set;
     auto launch = [&](auto kernel, int blocks, int first, int n) {
         return launch_tiles(kernel, blocks, smem_bytes<LPR, R, false>(), s, B.insts, B.tiles + first, n,
-                            B.counter, B.pubs, B.links, cur, toff, nsteps);
+                            B.nrules, B.counter, B.pubs, B.links, cur, toff, nsteps);
     };
     if constexpr (can_split(LPR, R)) {
         if (B.nrules > 0) {
@@ -1033,7 +1074,7 @@ cudaError_t launch_shape(const Lattice &L, const DevState &S, const TileDev &T, 
     auto launch = [&](auto kernel, int blocks, int first, int n) {
         return launch_tiles(kernel, blocks, smem_bytes<LPR, R, GRAD>(), s, T.map[cur],
                             static_cast<float *>(S.f[cur ^ 1]), static_cast<float4 *>(S.ucomp),
-                            (const uint8_t *)S.cls, T.tiles + first, n, T.counter, T.pubs, T.links,
+                            (const uint8_t *)S.cls, T.tiles + first, n, T.nrules, T.counter, T.pubs, T.links,
                             (const BCDev *)S.bcs, L, (const int64_t *)S.time, toff, nsteps, S.status);
     };
     if constexpr (can_split(LPR, R)) {

@@ -35,7 +35,7 @@ def _same(a, b):
 
 
 @pytest.mark.parametrize("at", [0, 1, 2, None], ids=["first", "second", "last", "three"])
-@pytest.mark.parametrize("side", [640], ids=["one_kernel"])
+@pytest.mark.parametrize("side", [640, 1100], ids=["one_kernel", "two_kernels"])
 def test_instance_without_material(side, at):
     """The one tile of a lattice without material has nothing to step; the block
     that takes it takes another tile behind it, of another instance (the batch
@@ -62,3 +62,34 @@ def test_instance_without_material(side, at):
             else:
                 assert _same(got, ref[id(w)][t]), (k, t)
     b.close()
+
+
+@pytest.mark.parametrize("lam", [1.0, 0.8], ids=["poisson", "nonpoisson"])
+def test_launches_of_two_kernels_on_two_streams(lam):
+    """Two handles whose launches are two kernels each, the second released by
+    the blocks of the first, stepped beside one another: every launch has its own
+    count of released blocks, back at zero when it ends."""
+    import torch
+    from paper_2208_04088_gb300 import _native as N
+    wls = [W.edge_crack(1300, 300, 0, lam_over_mu=lam, ny=1260),
+           W.hole_plate(1250, 1340, 130.5, 0, lam_over_mu=lam)]
+    ref = []
+    for w in wls:
+        s = N.Solver(_desc(w, time_block=1))
+        s.step(120)
+        s.sync()
+        ref.append(s.fields_host())
+        s.close()
+    ss = [N.Solver(_desc(w), stream=torch.cuda.Stream()) for w in wls]
+    before = [s.info()["kernel_launches"] for s in ss]
+    for n in (8, 5, 40, 64, 3):
+        for s in ss:
+            s.step(n)
+    for s, b in zip(ss, before):
+        s.sync()
+        # 120 steps: as many launches as chunks of them need, two kernels in each
+        assert s.info()["kernel_launches"] - b > 2 * (120 // s.info()["time_block"])
+        assert s.info()["time_block"] > 1
+    for s, r in zip(ss, ref):
+        assert _same(s.fields_host(), r)
+        s.close()
