@@ -548,24 +548,32 @@ __device__ __forceinline__ WallFrame wall_frame(const BLink &lk, const BCDev *__
 
 // Density deviation and Cauchy stress at the wall: the node's own values, or
 // the linear extrapolation along the link (1 + q) a(x) - q a(x - c_i) when
-// `neu_ex` (Sec. 4; q = 1/2 gives (3 a(x) - a(x - c_i))/2).
+// `neu_ex` (Sec. 4; q = 1/2 gives (3 a(x) - a(x - c_i))/2).  kSelect: both are
+// formed and one selected, without a branch.
 struct WallState {
     float drb, sxx, syy, sxy;
 };
 
+template <bool kSelect = false>
 __device__ __forceinline__ WallState wall_state(bool neu_ex, float q, float dr_x, float pxx_x,
                                                 float pyy_x, float pxy_x, float my_dr,
                                                 float my_xx, float my_yy, float my_xy,
                                                 const Lattice &L) {
     const float dvx = rmul(-L.lam_m_mu_r0, dr_x);
     const float sxx_x = radd(-pxx_x, dvx), syy_x = radd(-pyy_x, dvx), sxy_x = -pxy_x;
-    const float dvy = rmul(-L.lam_m_mu_r0, my_dr);
-    const float a1 = radd(1.0f, q);
-    const WallState e{rfma(a1, dr_x, -rmul(q, my_dr)), rfma(a1, sxx_x, -rmul(q, radd(-my_xx, dvy))),
-                      rfma(a1, syy_x, -rmul(q, radd(-my_yy, dvy))),
-                      rfma(a1, sxy_x, -rmul(q, -my_xy))};
-    return WallState{neu_ex ? e.drb : dr_x, neu_ex ? e.sxx : sxx_x, neu_ex ? e.syy : syy_x,
-                     neu_ex ? e.sxy : sxy_x};
+    WallState s{dr_x, sxx_x, syy_x, sxy_x};
+    if (kSelect || neu_ex) {
+        const float dvy = rmul(-L.lam_m_mu_r0, my_dr);
+        const float a1 = radd(1.0f, q);
+        const WallState e{rfma(a1, dr_x, -rmul(q, my_dr)),
+                          rfma(a1, sxx_x, -rmul(q, radd(-my_xx, dvy))),
+                          rfma(a1, syy_x, -rmul(q, radd(-my_yy, dvy))),
+                          rfma(a1, sxy_x, -rmul(q, -my_xy))};
+        if (!kSelect) return e;
+        s = WallState{neu_ex ? e.drb : s.drb, neu_ex ? e.sxx : s.sxx, neu_ex ? e.syy : s.syy,
+                      neu_ex ? e.sxy : s.sxy};
+    }
+    return s;
 }
 
 // The part of sigma* = t_n n n + t_t (n t + t n) + sigma_tt t t that the boundary
@@ -693,8 +701,8 @@ __device__ __forceinline__ float link_value(int k, const LinkRule &r, bool diric
                                             const Lattice &L) {
     // both rules, selected at the end: the links of a warp need not agree
     const float bb = rfma(r.fac, r.c0, rfma(r.kap, rsub(gy_i, gk), gi));
-    const WallState st = wall_state(neu_ex, r.q, dr_x, pxx_x, pyy_x, pxy_x, my_dr, my_xx, my_yy,
-                                    my_xy, L);
+    const WallState st = wall_state<true>(neu_ex, r.q, dr_x, pxx_x, pyy_x, pxy_x, my_dr, my_xx,
+                                          my_yy, my_xy, L);
     float sxx, syy, sxy;  // sigma* (Eq. trafocauchy)
     wall_sigma(r.t0, r.t1, WallData{r.c0, r.c1, r.c2}, st, sxx, syy, sxy);
     sxx = corner ? r.c0 : sxx;
@@ -711,8 +719,14 @@ __device__ __forceinline__ float cut_link_value(int k, bool miss, bool dirich, b
                                                 float my_yy, float my_xy,
                                                 const BCDev *__restrict__ bcs, float tb,
                                                 const Lattice &L) {
-    return link_value(k, link_rule(k, miss, dirich, corner, lk, bcs, tb, L), dirich, corner, neu_ex,
-                      gk, gi, gy_i, dr_x, pxx_x, pyy_x, pxy_x, my_dr, my_xx, my_yy, my_xy, L);
+    const LinkRule r = link_rule(k, miss, dirich, corner, lk, bcs, tb, L);
+    if (dirich) return rfma(r.fac, r.c0, rfma(r.kap, rsub(gy_i, gk), gi));
+    const WallState st = wall_state(neu_ex, r.q, dr_x, pxx_x, pyy_x, pxy_x, my_dr, my_xx, my_yy,
+                                    my_xy, L);
+    float sxx = r.c0, syy = r.c1, sxy = r.c2;
+    if (!corner) wall_sigma(r.t0, r.t1, WallData{r.c0, r.c1, r.c2}, st, sxx, syy, sxy);
+    const float eq = wall_equilibrium(k, wall_moments(st.drb, sxx, syy, sxy, L));
+    return anti_bounce_back(r.kap, r.fac, gk, gi, gy_i, eq);
 }
 
 // Populations f(x, t) of a boundary node: pulled where the link is intact,
