@@ -395,7 +395,9 @@ __device__ __forceinline__ bool tile_steps(const CUtensorMap *tf, float *__restr
                     fresh = (attr & kAttrRamp) != 0;
                 }
                 if (fresh) {
-                    rule = make_rule(links[rec.link0 + e], bcs, tb, L, attr);
+                    // tb is rounded twice where tb0 is no longer exact (2^24)
+                    const float at = tb0 < 16777216.0f ? tb : (float)(*time + toff - 1 + l);
+                    rule = make_rule(links[rec.link0 + e], bcs, at, L, attr);
                     if (mine_kept) {
                         my_rule = rule;
                     } else if (e < S::kRules) {
