@@ -1045,15 +1045,15 @@ cudaError_t batch_shape(const TileBatch &B, int cur, int toff, int nsteps, cudaS
         return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem_bytes<LPR, R, false>());
     };
-    static const cudaError_t attr_set = [&] {
+    if (B.ntiles <= 0) {
+        // at the creation of every batch: the limit is the current device's
         cudaError_t e = allow(k_tile_batch<LPR, R, SRC, Part::kAll>);
         if constexpr (can_split(LPR, R)) {
             if (e == cudaSuccess) e = allow(k_tile_batch<LPR, R, SRC, Part::kRules>);
             if (e == cudaSuccess) e = allow(k_tile_batch<LPR, R, SRC, Part::kInner>);
         }
         return e;
-    }();
-    if (attr_set != cudaSuccess || B.ntiles <= 0) return attr_set;
+    }
     auto launch = [&](auto kernel, int blocks, int first, int n) {
         return launch_tiles(kernel, blocks, smem_bytes<LPR, R, false>(), s, B.insts, B.tiles + first, n,
                             B.nrules, B.counter, B.pubs, B.links, cur, toff, nsteps);
