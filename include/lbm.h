@@ -214,9 +214,10 @@ lbm_status lbm_geom_build(const lbm_geom *geom, uint8_t *node_type, lbm_link *li
 
 /* Device bytes a handle for `desc` needs (distributions, displacement,
  * tables, field staging).  Host tables are validated as in lbm_create.  The
- * tables of the register tiles come on top: lbm_create allocates them itself
- * (about 100 bytes per boundary node and 32 per tile) and, if it cannot, steps
- * in strips (lambda = mu, large lattices) or one step per launch. */
+ * tables of the register tiles (about 100 bytes per boundary node and 32 per
+ * tile) lie in it for lambda = mu lattices large enough for strips; for the
+ * others they come on top: lbm_create allocates them itself and, if it cannot,
+ * steps one step per launch. */
 lbm_status lbm_workspace_size(const lbm_desc *desc, uint64_t *bytes);
 
 /* Create a solver: validates and classifies the tables on the host, copies

@@ -264,9 +264,10 @@ cudaError_t host_buffers(lbm_solver *h) {
 }
 
 // Register tiles for a handle whose state is allocated: the plan, and its
-// tables in memory of the handle's own.  Without that memory the handle keeps
-// the stepping form its workspace was laid out for.
-static cudaError_t tile_create(lbm_solver *h) {
+// tables in `spare` (the workspace's part for strips, which tiles leave idle)
+// or, where it is too small or absent, in memory of the handle's own.  Without
+// that memory the handle keeps the stepping form its workspace was laid out for.
+static cudaError_t tile_create(lbm_solver *h, char *spare, size_t spare_bytes) {
     if (!tile_supported()) return cudaSuccess;
     TilePlan plan;
     tile_choose(h->tab, h->L.grad != 0, h->L.wall_node != 0, device_sms(), &plan);
@@ -275,12 +276,13 @@ static cudaError_t tile_create(lbm_solver *h) {
     const size_t bp = align256(plan.pubs.size() * sizeof(uint32_t));
     const size_t bl = align256(plan.links.size() * sizeof(TileLink));
     TileDev &T = h->tile;
-    if (cudaMalloc(&T.mem, bt + bp + bl + 256) != cudaSuccess) {
+    const size_t need = bt + bp + bl + 256;
+    if (need > spare_bytes && cudaMalloc(&T.mem, need) != cudaSuccess) {
         cudaGetLastError();
         T.mem = nullptr;
         return cudaSuccess;
     }
-    char *m = static_cast<char *>(T.mem);
+    char *m = T.mem ? static_cast<char *>(T.mem) : spare;
     T.tiles = reinterpret_cast<const TileRec *>(m);
     T.pubs = reinterpret_cast<const uint32_t *>(m + bt);
     T.links = reinterpret_cast<const TileLink *>(m + bt + bp);
@@ -415,7 +417,7 @@ lbm_status create_prepared(const lbm_desc *desc, Tables &&tab, const Units &unit
     // steps of the crack in 171 us against 359 (strips: 349).
     if (e == cudaSuccess && desc->time_block == 0 &&
         h->storage == LBM_F32 && !in_place)
-        e = tile_create(h);
+        e = tile_create(h, b + lay.nw, h->block > 1 ? lay.total - lay.nw : 0);
     if (e == cudaSuccess && h->block > 1 && h->tile.shape < 0) {
         if (!wave_supported(h->L)) {
             if (desc->time_block == LBM_TIME_BLOCK) {

@@ -310,7 +310,8 @@ bool tile_plan(const Tables &t, bool wall_node, int shape, TilePlan *p);
 // p->shape is -1 where one step per launch is modelled to be faster.
 void tile_choose(const Tables &t, bool grad, bool wall_node, int sms, TilePlan *p);
 
-// Device side of a plan (tables owned by the handle, outside its workspace).
+// Device side of a plan; its tables lie in the workspace's part for strips, or
+// in `mem`, which the handle owns.
 struct TileDev {
     CUtensorMap map[2];  // the population buffers, box of one tile
     int shape = -1, ntiles = 0, sms = 1;
