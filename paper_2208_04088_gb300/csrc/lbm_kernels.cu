@@ -27,13 +27,10 @@
 namespace lbm {
 // ---------------------------------------------------------------------------
 // Kernels.
-// Blocks of 128 x 2 threads: one step in place of the 2048^2 crack 74.5 us, with
-// 64 x 4 75.0, with 32 x 8 76.4 (a block then touches fewer, longer runs of
-// every population plane).
-constexpr int kBX = 128, kBY = 2;
+constexpr int kBT = 256;  // most threads of a block of the lattice kernels (one node or pair each)
 constexpr int kBB = 64;  // threads per block of the boundary-list kernels
 
-// Interior kernel: one node per thread (NR rows per thread, kBY rows apart).
+// Interior kernel: one node per thread.
 // Every load of a node -- the nine pulled populations and the displacement
 // record -- is issued before any arithmetic, so all of them are in flight
 // together.
@@ -51,37 +48,28 @@ __device__ __forceinline__ int64_t scales_of_step(Lattice &L, const int64_t *tim
     return t;
 }
 
-template <class T, int NR, int LAY = kPull>
-__global__ void __launch_bounds__(kBX *kBY, 8) k_interior(const T *src, T *dst,
+template <class T, int LAY = kPull>
+__global__ void __launch_bounds__(kBT, 8) k_interior(const T *src, T *dst,
                                                        URec<T> *__restrict__ uc,
                                                        const uint8_t *__restrict__ cls,
                                                        const float *__restrict__ rho, Lattice L,
                                                        uint32_t *__restrict__ status,
                                                        const int64_t *__restrict__ time, int toff) {
-    const int x = blockIdx.x * kBX + threadIdx.x;
-    const int y0 = blockIdx.y * (kBY * NR) + threadIdx.y;
-    scales_of_step<T>(L, time, toff, x == 0 && y0 == 0);
-    if (x >= L.nx) return;
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        const int y = y0 + r * kBY;
-        if (y < L.ny)
-            interior_node<T, LAY>(src, dst, uc, cls, rho, L, (int64_t)y * L.pitch + x, status);
-    }
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    scales_of_step<T>(L, time, toff, x == 0 && y == 0);
+    if (x < L.nx && y < L.ny)
+        interior_node<T, LAY>(src, dst, uc, cls, rho, L, (int64_t)y * L.pitch + x, status);
 }
 
 // 16-bit storage, two buffers, lambda = mu: two adjacent nodes per thread
-// (interior_pair).  Threads per SM the register bound aims at: FP16 measured fastest at 1536 (40
-// registers: 93.9 against 90.4 GLUPS at 1024 on the 2048^2 crack), BF16 at 1024
-// (100.7 against 98.9 at 1536).  Blocks of 64 threads in one row: 21.6 ms for
-// 500 steps of the FP16 crack, 21.9 with 128, 22.5 with 128 x 2, 23.0 with
-// 32 x 8 (longer runs of every plane, and the next block placed as soon as two
-// warps end).
-template <class T> constexpr int kPairMinBlocks = std::is_same<T, __half>::value ? 24 : 16;
-constexpr int kPX = 64;  // threads of its blocks, all in one row
+// (interior_pair).  Blocks of kBT threads the register bound aims at: FP16
+// measured fastest at six (40 registers: 93.9 against 90.4 GLUPS at four on the
+// 2048^2 crack), BF16 at four (100.7 against 98.9 at six).
+template <class T> constexpr int kPairMinBlocks = std::is_same<T, __half>::value ? 6 : 4;
 
 template <class T>
-__global__ void __launch_bounds__(kPX, kPairMinBlocks<T>) k_interior_pair(const T *__restrict__ src,
+__global__ void __launch_bounds__(kBT, kPairMinBlocks<T>) k_interior_pair(const T *__restrict__ src,
                                                             T *__restrict__ dst,
                                                             float2 *__restrict__ uc,
                                                             const uint8_t *__restrict__ cls,
@@ -89,8 +77,8 @@ __global__ void __launch_bounds__(kPX, kPairMinBlocks<T>) k_interior_pair(const 
                                                             uint32_t *__restrict__ status,
                                                             const int64_t *__restrict__ time,
                                                             int toff) {
-    const int x0 = 2 * (int)(blockIdx.x * kPX + threadIdx.x);
-    const int y = blockIdx.y + threadIdx.y;  // threadIdx.y = 0
+    const int x0 = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
     // FP16: this step's scales.  The thread of node (0, 0), which is never
     // interior, publishes them after its node classes have been read, so that
     // no store sits between the loads of a thread and delays them.
@@ -244,13 +232,13 @@ __global__ void __launch_bounds__(kBB) k_boundary_scatter(const float *__restric
 // boundary rules at boundary nodes.  Writes the deviation rho - rho0 into a
 // dense [ny][pitch] array.
 template <class T>
-__global__ void __launch_bounds__(kBX *kBY) k_density_interior(const T *__restrict__ src,
+__global__ void __launch_bounds__(kBT) k_density_interior(const T *__restrict__ src,
                                                                const uint8_t *__restrict__ cls,
                                                                float *__restrict__ rho, Lattice L,
                                                                const int64_t *__restrict__ time) {
     scales_of_step<T>(L, time, 0, false);
-    const int x = blockIdx.x * kBX + threadIdx.x;
-    const int y = blockIdx.y * kBY + threadIdx.y;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= L.nx || y >= L.ny) return;
     const int64_t k = (int64_t)y * L.pitch + x;
     if (cls[k] != kInterior) return;
@@ -299,15 +287,15 @@ __device__ __forceinline__ void write_fields(float *__restrict__ out, int64_t N,
 }
 
 template <class T, int LAY = kPull>
-__global__ void __launch_bounds__(kBX *kBY) k_fields_interior(const T *__restrict__ src,
+__global__ void __launch_bounds__(kBT) k_fields_interior(const T *__restrict__ src,
                                                               const URec<T> *__restrict__ uc,
                                                               const uint8_t *__restrict__ cls,
                                                               const float *__restrict__ rho,
                                                               Lattice L, float *__restrict__ out,
                                                               const int64_t *__restrict__ time) {
     scales_of_step<T>(L, time, 0, false);  // the populations stored by the last step
-    const int x = blockIdx.x * kBX + threadIdx.x;
-    const int y = blockIdx.y * kBY + threadIdx.y;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= L.nx || y >= L.ny) return;
     const int64_t k = (int64_t)y * L.pitch + x;
     const int64_t N = (int64_t)L.nx * L.ny, o = (int64_t)y * L.nx + x;
@@ -406,6 +394,31 @@ static cudaError_t launch_boundary(const T *src, T *dst, const DevState &S, cons
                               (const int64_t *)S.time, toff, S.status, stage);
 }
 
+// The blocks of `blk` threads, `per` nodes in a row to each, that cover the lattice.
+static dim3 lattice_grid(const Lattice &L, int per, dim3 blk) {
+    const int w = per * (int)blk.x;
+    return dim3((L.nx + w - 1) / w, (L.ny + (int)blk.y - 1) / (int)blk.y);
+}
+
+// Blocks of one node per thread.  Long rows touch fewer, longer runs of every
+// population plane, which pays where the planes come from HBM; a small lattice
+// is bound by latency, and short rows idle less at its right edge.  Us a step,
+// 32 x 4 / 128 x 2 threads, plates with a hole: in place 140 x 400 6.64 / 6.85,
+// 400^2 7.74 / 8.13, 512^2 9.18 / 9.12, 640^2 10.50 / 10.28, 2048^2 73.5 / 71.5;
+// two buffers 520 x 1000 6.64 / 6.92, 800^2 7.34 / 7.50, 1024^2 12.53 / 12.41.
+static dim3 node_block(const Lattice &L) {
+    const int64_t nodes = (int64_t)L.nx * L.ny;
+    return L.nx >= 512 && nodes >= (L.in_place ? 1 << 18 : 1 << 20) ? dim3(128, 2) : dim3(32, 4);
+}
+// Blocks of two nodes per thread (16-bit storage): 64 x 1 beyond L2, where the
+// next block also finds its place as soon as two warps end.  32 x 4 / 64 x 1,
+// FP16: 520 x 1000 7.04 / 7.63, 800^2 7.68 / 8.03, 1024^2 10.05 / 10.12, 1400^2
+// 17.30 / 17.17, 2048^2 43.3 / 42.7 (32 x 8 44.4); BF16: 520 x 1000 5.98 / 6.42,
+// 1024^2 8.56 / 8.66, 1400^2 14.70 / 14.63, 2048^2 40.0 / 39.4.
+static dim3 pair_block(const Lattice &L) {
+    return L.nx >= 1024 && (int64_t)L.nx * L.ny > 1 << 20 ? dim3(64, 1) : dim3(32, 4);
+}
+
 template <class T>
 static void launch_interior(const T *src, T *dst, const DevState &S, const Lattice &L, int toff,
                             cudaStream_t s) {
@@ -418,18 +431,16 @@ static void launch_interior(const T *src, T *dst, const DevState &S, const Latti
     }
     if constexpr (!std::is_same<T, float>::value) {
         // 16-bit storage: two nodes per thread
-        const dim3 grd((L.nx + 2 * kPX - 1) / (2 * kPX), L.ny);
-        k_interior_pair<T><<<grd, kPX, 0, s>>>(src, dst, static_cast<float2 *>(S.ucomp), S.cls, L,
-                                               S.status, S.time, toff);
+        const dim3 blk = pair_block(L);
+        k_interior_pair<T><<<lattice_grid(L, 2, blk), blk, 0, s>>>(
+            src, dst, static_cast<float2 *>(S.ucomp), S.cls, L, S.status, S.time, toff);
         return;
     }
     // one row per thread measured fastest for every storage (2 and 4 rows cost
     // occupancy: 58+ registers)
-    constexpr int NR = 1;
-    const dim3 blk(kBX, kBY), grd((L.nx + kBX - 1) / kBX, (L.ny + kBY * NR - 1) / (kBY * NR));
-    k_interior<T, NR><<<grd, blk, 0, s>>>(src, dst, static_cast<URec<T> *>(S.ucomp), S.cls, S.rho,
-                                          L, S.status, S.time,
-                                          toff);
+    const dim3 blk = node_block(L);
+    k_interior<T><<<lattice_grid(L, 1, blk), blk, 0, s>>>(src, dst, static_cast<URec<T> *>(S.ucomp),
+                                                          S.cls, S.rho, L, S.status, S.time, toff);
 }
 
 // In-place step of parity LAY: every boundary node reads its inputs and
@@ -457,8 +468,8 @@ static cudaError_t step_in_place(const Lattice &L, const DevState &S, int toff,
         cudaEventRecord(join, s_side);
     }
     if (ev) cudaEventRecord(ev->before_interior, s_main);
-    const dim3 blk(kBX, kBY), grd((L.nx + kBX - 1) / kBX, (L.ny + kBY - 1) / kBY);
-    k_interior<T, 1, LAY><<<grd, blk, 0, s_main>>>(f, f, static_cast<URec<T> *>(S.ucomp), S.cls,
+    const dim3 blk = node_block(L), grd = lattice_grid(L, 1, blk);
+    k_interior<T, LAY><<<grd, blk, 0, s_main>>>(f, f, static_cast<URec<T> *>(S.ucomp), S.cls,
                                                    S.rho, L, S.status, S.time,
                                                    toff);
     if (ev) cudaEventRecord(ev->after_interior, s_main);
@@ -478,7 +489,7 @@ static cudaError_t step_t(const Lattice &L, const DevState &S, int cur, int toff
                    : step_in_place<T, kAAEven>(L, S, toff, s_main, s_side, fork, join, ev);
     const T *src = static_cast<const T *>(S.f[cur]);
     T *dst = static_cast<T *>(S.f[cur ^ 1]);
-    const dim3 blk(kBX, kBY), grd((L.nx + kBX - 1) / kBX, (L.ny + kBY - 1) / kBY);
+    const dim3 blk = node_block(L), grd = lattice_grid(L, 1, blk);
     const int nbb = (L.nb + kBB - 1) / kBB;
     // lambda != mu: densities of the boundary nodes first (the interior kernel
     // forms all other densities it needs in shared memory)
@@ -534,7 +545,7 @@ cudaError_t launch_advance(const DevState &S, int64_t n, cudaStream_t s) {
 template <class T, int LAY>
 static void fields_in_place(const Lattice &L, const DevState &S, cudaStream_t s) {
     const T *src = static_cast<const T *>(S.f[0]);
-    const dim3 blk(kBX, kBY), grd((L.nx + kBX - 1) / kBX, (L.ny + kBY - 1) / kBY);
+    const dim3 blk = node_block(L), grd = lattice_grid(L, 1, blk);
     k_fields_interior<T, LAY><<<grd, blk, 0, s>>>(src, static_cast<const URec<T> *>(S.ucomp), S.cls,
                                                   S.rho, L, S.stage, S.time);
     if (L.nb > 0)
@@ -553,7 +564,7 @@ static cudaError_t fields_t(const Lattice &L, const DevState &S, int cur, cudaSt
         return cudaGetLastError();
     }
     const T *src = static_cast<const T *>(S.f[cur]);
-    const dim3 blk(kBX, kBY), grd((L.nx + kBX - 1) / kBX, (L.ny + kBY - 1) / kBY);
+    const dim3 blk = node_block(L), grd = lattice_grid(L, 1, blk);
     const int nbb = (L.nb + kBB - 1) / kBB;
     if (L.grad) {
         k_density_interior<T><<<grd, blk, 0, s>>>(src, S.cls, S.rho, L, S.time);
