@@ -579,13 +579,50 @@ lbm_status build_tile_tables(lbm_engine *E) {
     return LBM_OK;
 }
 
+bool steps_in_place(const lbm_engine *E) {
+    bool any = false;
+    for (const auto &I : E->inst) any = any || (!I.blocked && I.h->L.in_place);
+    return any;
+}
+
+// Nodes per tile row: two per thread when the pull-only 16-bit form runs.
+int tile_nodes_x(const lbm_engine *E) {
+    return (E->storage != LBM_F32 && !steps_in_place(E) ? 2 : 1) * E->shape.tile_x;
+}
+
+// The shape a lockstep batch starts with (lbm_batch_tune measures others).  It
+// keeps its tiles, so its grid can follow them: one block per 32 x 4 tile, or,
+// where the tiles fill the device many times over, one per run of four, which
+// stages an instance's descriptor once.  A run is a serial chain, so few tiles
+// are better off alone, and longer in place, where every tile comes between
+// the staging of the boundary and its scatter.  Us a step in runs / one by one /
+// in the persistent grid of 32 x 8 that the server keeps: FP16 3 of 128^2 (1 tile
+// per SM) 14.6 / 14.1 / 14.0, 3 of 256^2 (5) 15.0 / 15.0 / 15.1, 24 of 100^2 (8)
+// 15.9 / 16.1 / 16.3, 40 of 256^2 (67) 47.0 / 57.5 / 50.3; FP32 24 of 64^2 (5)
+// 13.6 / 13.5 / 13.6, 24 of 100^2 (16) 14.5 / 14.9 / 14.6; in place 3 of 64^2
+// (0.6) 14.6 / 10.9 / 10.5, 3 of 128^2 (2.5) 15.1 / 10.8 / 11.0, 24 of 100^2 (16)
+// 20.2 / 18.0 / 18.3, 4 of 512^2 (54) 27.0 / 24.3 / 26.6, 40 of 256^2 (135)
+// 89.0 / 88.1 / 93.8, 16 of 512^2 (216) 110.8 / 111.6 / 118.5.
+constexpr int kRunTiles = 8, kRunTilesInPlace = 144;  // tiles per SM from which runs pay
+constexpr int kGridTilesInPlace = 2;                  // below which the persistent grid does
+
+void batch_shape(lbm_engine *E) {
+    E->shape = {32, 4, 16, 2};
+    int64_t tiles = 0;
+    for (const Instance &I : E->inst)
+        if (!I.blocked)
+            tiles += (int64_t)((I.h->L.nx + tile_nodes_x(E) - 1) / tile_nodes_x(E)) *
+                     ((I.h->L.ny + E->shape.tile_y - 1) / E->shape.tile_y);
+    const bool in_place = steps_in_place(E);
+    if (tiles >= (int64_t)(in_place ? kRunTilesInPlace : kRunTiles) * E->sms)
+        E->shape.dynamic = 3;
+    else if (in_place && tiles < (int64_t)kGridTilesInPlace * E->sms)
+        E->shape = {32, 8, 8, 0};
+}
+
 // Rebuild the instance, tile and boundary-node tables on the device.
 lbm_status rebuild_tables(lbm_engine *E) {
-    const int TX = E->shape.tile_x, TY = E->shape.tile_y;
-    // nodes per tile row: two per thread when the pull-only 16-bit form runs
-    bool any_in_place = false;
-    for (const auto &I : E->inst) any_in_place = any_in_place || (!I.blocked && I.h->L.in_place);
-    const int TXN = (E->storage != LBM_F32 && !any_in_place) ? 2 * TX : TX;
+    const int TY = E->shape.tile_y, TXN = tile_nodes_x(E);
     std::vector<InstDev> hi(E->inst.size());
     std::vector<int2> tiles, bmap, simple;
     for (size_t i = 0; i < E->inst.size(); ++i) {
@@ -1101,12 +1138,6 @@ extern "C" lbm_status lbm_batch_create(const lbm_desc *descs, int32_t count, voi
     std::unique_ptr<lbm_engine> E(new lbm_engine());
     lbm_status st = engine_init(E.get(), descs[0].storage, stream);
     if (st != LBM_OK) return st;
-    // A lockstep batch keeps its tiles, so its grid can follow them: runs of
-    // four small tiles per block stage an instance's descriptor once per run
-    // and leave the order to the block scheduler (40 FP16 plates with holes,
-    // 256 steps: 42.3 ms; 46.8 with one tile per block, 50.7 with the
-    // persistent grid, which the server keeps).
-    E->shape = {32, 4, 16, 3};
     uint64_t total = 0;
     for (int32_t i = 0; i < count; ++i) {
         uint64_t b = 0;
@@ -1121,6 +1152,7 @@ extern "C" lbm_status lbm_batch_create(const lbm_desc *descs, int32_t count, voi
         st = admit(E.get(), descs[i], i, INT64_MAX);
         if (st != LBM_OK) return st;
     }
+    batch_shape(E.get());
     st = rebuild_tables(E.get());
     if (st != LBM_OK) return st;
     *out = E.release();

@@ -36,3 +36,20 @@ def test_one_lattice(nx, ny, storage):
     wl = _plate(nx, ny)
     two = _fields(N.desc_from_workload(wl, storage=storage, time_block=1), 37)
     _same(two, _fields(N.desc_from_workload(wl, storage=storage, in_place=True), 37))
+
+
+@pytest.mark.parametrize("form", ["f32", "bf16", "in_place"])
+@pytest.mark.parametrize("count,nx,ny", [(2, 50, 41), (9, 100, 101), (25, 100, 101), (60, 100, 101), (260, 100, 101)])
+def test_batch(count, nx, ny, form):
+    """Batches stepped one step per launch, from less than a tile per SM to more
+    than 144: one block per tile, per run of four, and the persistent grid."""
+    from paper_2208_04088_gb300 import _native as N
+    kw = dict(in_place=True) if form == "in_place" else dict(storage=form)
+    wl = _plate(nx, ny)
+    b = N.Batch([N.desc_from_workload(wl, **kw) for _ in range(count)])
+    b.step(37)
+    b.sync()
+    alone = _fields(N.desc_from_workload(wl, time_block=0 if form == "in_place" else 1, **kw), 37)
+    for i in {0, count // 2, count - 1}:
+        _same(b.fields_host(i), alone)
+    b.close()
