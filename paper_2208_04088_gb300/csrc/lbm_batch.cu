@@ -1190,7 +1190,7 @@ extern "C" lbm_status lbm_batch_set_shape(lbm_batch b, const lbm_launch_shape *s
     if (!ok_tile || shape->blocks_per_sm < 1 || shape->blocks_per_sm > 64 ||
         shape->dynamic < 0 || shape->dynamic > 3) {
         set_error("lbm_batch_set_shape: tiles 32x4, 32x8, 32x16 or 64x4; 1..64 blocks per SM; "
-                  "schedule 0, 1 or 2");
+                  "schedule 0 to 3");
         return LBM_ERR_ARG;
     }
     b->shape = *shape;
