@@ -38,11 +38,11 @@ sys.path.insert(0, ROOT)
 
 METRIC = "GLUPS (giga lattice updates per second, whole job)"
 # FP32 operations of one lattice update in the temporally blocked kernels (FMA =
-# 2): moments and populations 39, 13 of them FMAs, displacement update 11
-FLOPS_PER_UPDATE = 63
+# 2): moments and populations 42, 9 of them FMAs, displacement update 11
+FLOPS_PER_UPDATE = 62
 # with lambda != mu also the source from the density gradient (10) and its eight
 # FMAs in the collision
-FLOPS_PER_UPDATE_GRAD = 89
+FLOPS_PER_UPDATE_GRAD = 88
 # the kernel sources each kernel's recorded DRAM traffic depends on
 KERNEL_SOURCES = {"k_interior": ("lbm_kernels.cu", "lbm_device.cuh"),
                   "k_interior_pair": ("lbm_kernels.cu", "lbm_device.cuh", "lbm_pair.cuh"),

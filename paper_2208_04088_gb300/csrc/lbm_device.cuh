@@ -165,7 +165,7 @@ template <> __device__ __forceinline__ F2 splat<F2>(float c) { return f2(c, c); 
 
 // ---------------------------------------------------------------------------
 // The arithmetic of a storage form.  The two evaluate the same collision with
-// different rounding orders: kSums32 needs 39 operations per node without a
+// different rounding orders: kSums32 needs 42 operations per node without a
 // source, kSums16 65.  16-bit storage keeps the longer one: a stored value that
 // rounds the other way would move its results by their own error (1e-3).
 enum : int { kSums16 = 0, kSums32 = 1 };
@@ -180,23 +180,28 @@ template <class V> struct RawT {
 };
 using Raw = RawT<float>;
 
-// kSums32: every sum of three takes the sum of its outer two, so a 1-D map is
-// three operations.
-template <class V> __device__ __forceinline__ RawT<V> raw_sums(const V f[9]) {
-    // rows c_y = -1: (f7, f4, f8); c_y = 0: (f3, f0, f1); c_y = +1: (f6, f2, f5)
-    const V a2 = radd(f[8], f[7]), a1 = rsub(f[8], f[7]), a0 = radd(a2, f[4]);
-    const V b2 = radd(f[1], f[3]), b1 = rsub(f[1], f[3]), b0 = radd(b2, f[0]);
-    const V c2 = radd(f[5], f[6]), c1 = rsub(f[5], f[6]), c0 = radd(c2, f[2]);
+// kSums32: the moments from the sums of the outer columns (c_x = +1, -1) and rows
+// (c_y = +1, -1), which the collision needs again.
+template <class V> struct SumsT {
+    V east, west, north, south;
+};
+template <class V> __device__ __forceinline__ RawT<V> raw_sums(const V f[9], SumsT<V> &s) {
+    const V e = radd(f[5], f[8]), w = radd(f[6], f[7]);  // corners of each side
+    const V n = radd(f[5], f[6]), o = radd(f[8], f[7]);
+    s.east = radd(f[1], e);
+    s.west = radd(f[3], w);
+    s.north = radd(f[2], n);
+    s.south = radd(f[4], o);
     RawT<V> m;
-    m.m02 = radd(c0, a0);
-    m.m00 = radd(m.m02, b0);
-    m.m01 = rsub(c0, a0);
-    m.m12 = radd(c1, a1);
-    m.m10 = radd(m.m12, b1);
-    m.m11 = rsub(c1, a1);
-    m.m22 = radd(c2, a2);
-    m.m20 = radd(m.m22, b2);
-    m.m21 = rsub(c2, a2);
+    m.m20 = radd(s.east, s.west);
+    m.m10 = rsub(s.east, s.west);
+    m.m02 = radd(s.north, s.south);
+    m.m01 = rsub(s.north, s.south);
+    m.m00 = radd(m.m20, radd(radd(f[2], f[4]), f[0]));
+    m.m22 = radd(n, o);
+    m.m21 = rsub(n, o);
+    m.m12 = rsub(e, w);
+    m.m11 = rsub(rsub(f[5], f[6]), rsub(f[8], f[7]));
     return m;
 }
 
@@ -248,8 +253,9 @@ struct Mom {
 
 template <int kSums> __device__ __forceinline__ Mom moments(const float f[9]) {
     Raw r;
+    SumsT<float> s;
     if constexpr (kSums == kSums32)
-        r = raw_sums(f);
+        r = raw_sums(f, s);
     else
         r = raw_moments(f);
     return Mom{r.m00, r.m10, r.m01, r.m20, r.m02, r.m11};
@@ -294,18 +300,23 @@ __device__ __forceinline__ void collide_v(V f[9], V sx, V sy, V w, V s3, V &dr_o
 }
 
 // kSums32: the collision changes only the moments m_xxy, m_xyy and m_xxyy (and j
-// by the source), so it is f plus the inverse transforms of those three
-// changes, formed from their negatives n = m - m^eq: corners take -omega/4 of
-// n_xxyy +- n_xxy +- n_xyy, the axis directions +omega/2 of n_xxyy +- their odd
-// one, the rest population -omega n_xxyy.  The factors are exact multiples of
-// one rounded omega, so rho, j and P lose nothing to them.  kSource: S enters
-// j, the odd moments with (1 - 1/(2 tau))/3 and the axis directions with S/2;
-// without it the operations whose result S = 0 leaves unchanged are left out.
+// by the source).  The corners take -omega/4 of n_xxyy +- n_xxy +- n_xyy, n = m -
+// m^eq, the rest population -omega n_xxyy.  The sums of the outer columns and
+// rows stay as they were (but for the source), so an axis direction is its sum
+// less the two corners just formed: what rounding adds to a corner it takes off
+// the axes, and j, whose errors a whole wave front shares and the displacement
+// adds up, drifts by an axis population's rounding alone.  (Increments of
+// +omega/2 (n_xxyy +- n) for the axes need three operations less, 2048^2 crack
+// 11.42 ms against 11.66, but each population then rounds by itself: relative
+// error against 64 bits over eight loads of that crack 2.6e-7 to 6.1e-7, here 2.5e-7
+// to 2.7e-7, kSums16's order 3.1e-7 to 4.0e-7.)  kSource: S enters j, the odd
+// moments with (1 - 1/(2 tau))/3 and the outer sums with S/2; without it the
+// operations whose result S = 0 leaves unchanged are left out.
 template <class V> struct Relax {
-    V w, w2, mw4, msrc;  // -omega, omega/2, -omega/4, -(tau - 1/2)/3
+    V w, mw4, msrc;  // -omega, -omega/4, -(tau - 1/2)/3
 };
 template <class V> __device__ __forceinline__ Relax<V> relax_of(const Lattice &L) {
-    return Relax<V>{splat<V>(-L.omega), splat<V>(rmul(0.5f, L.omega)), splat<V>(rmul(-0.25f, L.omega)),
+    return Relax<V>{splat<V>(-L.omega), splat<V>(rmul(-0.25f, L.omega)),
                     splat<V>(-L.src_tau)};
 }
 
@@ -313,16 +324,17 @@ template <bool kSource, class V>
 __device__ __forceinline__ void collide_sums(V f[9], V sx, V sy, const Relax<V> &c, V &dr_out, V &jx_out,
                                              V &jy_out) {
     const V mthird = splat<V>(-1.0f / 3.0f);
-    const RawT<V> m = raw_sums(f);
+    SumsT<V> s;
+    const RawT<V> m = raw_sums(f, s);
     V jx = m.m10, jy = m.m01;
     if constexpr (kSource) {
         const V half = splat<V>(0.5f), mhalf = splat<V>(-0.5f);
         jx = rfma(half, sx, jx);
         jy = rfma(half, sy, jy);
-        f[1] = rfma(half, sx, f[1]);
-        f[3] = rfma(mhalf, sx, f[3]);
-        f[2] = rfma(half, sy, f[2]);
-        f[4] = rfma(mhalf, sy, f[4]);
+        s.east = rfma(half, sx, s.east);
+        s.west = rfma(mhalf, sx, s.west);
+        s.north = rfma(half, sy, s.north);
+        s.south = rfma(mhalf, sy, s.south);
     }
     V n21 = rfma(jy, mthird, m.m21), n12 = rfma(jx, mthird, m.m12);
     if constexpr (kSource) {
@@ -335,10 +347,10 @@ __device__ __forceinline__ void collide_sums(V f[9], V sx, V sy, const Relax<V> 
     f[6] = rfma(c.mw4, rsub(p, n12), f[6]);
     f[7] = rfma(c.mw4, rsub(q, n12), f[7]);
     f[8] = rfma(c.mw4, radd(q, n12), f[8]);
-    f[1] = rfma(c.w2, radd(n22, n12), f[1]);
-    f[3] = rfma(c.w2, rsub(n22, n12), f[3]);
-    f[2] = rfma(c.w2, p, f[2]);
-    f[4] = rfma(c.w2, q, f[4]);
+    f[1] = rsub(s.east, radd(f[5], f[8]));
+    f[3] = rsub(s.west, radd(f[6], f[7]));
+    f[2] = rsub(s.north, radd(f[5], f[6]));
+    f[4] = rsub(s.south, radd(f[8], f[7]));
     f[0] = rfma(c.w, n22, f[0]);
     dr_out = m.m00;
     jx_out = jx;
@@ -875,10 +887,8 @@ __device__ __forceinline__ float boundary8_collide(float fk, float g0, int kdir,
 // Density deviation rho - rho0 of nine populations, summed as raw_sums forms
 // m00 (so it equals moments<kSums32>(f).dr bit for bit); one node or two.
 template <class V> __device__ __forceinline__ V density_of(const V f[9]) {
-    const V a0 = radd(radd(f[8], f[7]), f[4]);
-    const V b0 = radd(radd(f[1], f[3]), f[0]);
-    const V c0 = radd(radd(f[5], f[6]), f[2]);
-    return radd(radd(c0, a0), b0);
+    const V east = radd(f[1], radd(f[5], f[8])), west = radd(f[3], radd(f[6], f[7]));
+    return radd(radd(east, west), radd(radd(f[2], f[4]), f[0]));
 }
 
 // The source coefficient (mu - lambda)/rho = (mu - lambda) times an

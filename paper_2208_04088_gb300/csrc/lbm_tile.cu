@@ -25,7 +25,7 @@
 // block's warps meet at a split barrier.  Tiles with them take tile_steps.
 //
 // What bounds it: instruction issue in the tiles of a large lattice (a 64 x 64
-// tile updates 4096 nodes per step, 39 paired operations per pair and 7 paired
+// tile updates 4096 nodes per step, 42 paired operations per pair and 7 paired
 // ones per node for the displacement, of which the core's 48 x 48 count; about
 // as many moves, shuffles and address operations go with them).  One interior
 // 64 x 64 tile, 8 steps: 14 us, of which 1.3 us a step (1350 cycles of FP32
