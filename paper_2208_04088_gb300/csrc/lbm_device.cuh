@@ -731,14 +731,29 @@ __device__ __forceinline__ float cut_link_value(int k, bool miss, bool dirich, b
                                                 float my_yy, float my_xy,
                                                 const BCDev *__restrict__ bcs, float tb,
                                                 const Lattice &L) {
-    const LinkRule r = link_rule(k, miss, dirich, corner, lk, bcs, tb, L);
-    if (dirich) return rfma(r.fac, r.c0, rfma(r.kap, rsub(gy_i, gk), gi));
-    const WallState st = wall_state(neu_ex, r.q, dr_x, pxx_x, pyy_x, pxy_x, my_dr, my_xx, my_yy,
+    const float q = miss ? 0.5f : lk.q;
+    float kap, fac;
+    link_kappa(q, kap, fac);
+    if (dirich) {
+        float jsx, jsy;
+        dirichlet_momentum(lk, bcs, tb, L, jsx, jsy);
+        return bounce_back(k, kap, fac, gk, gi, gy_i, jsx, jsy);
+    }
+    const WallState st = wall_state(neu_ex, q, dr_x, pxx_x, pyy_x, pxy_x, my_dr, my_xx, my_yy,
                                     my_xy, L);
-    float sxx = r.c0, syy = r.c1, sxy = r.c2;
-    if (!corner) wall_sigma(r.t0, r.t1, WallData{r.c0, r.c1, r.c2}, st, sxx, syy, sxy);
+    float sxx, syy, sxy;  // sigma* (Eq. trafocauchy)
+    if (corner) {
+        float tax, tay, tbx, tby;
+        traction(bcs[lk.bc], lk.n0, 0.0f, tb, tax, tay);
+        traction(bcs[lk.bc2], 0.0f, lk.n1, tb, tbx, tby);
+        sxx = rmul(tax, lk.n0);
+        syy = rmul(tby, lk.n1);
+        sxy = rmul(0.5f, rfma(tay, lk.n0, rmul(tbx, lk.n1)));
+    } else {
+        wall_sigma(wall_frame(lk, bcs, tb), st, sxx, syy, sxy);
+    }
     const float eq = wall_equilibrium(k, wall_moments(st.drb, sxx, syy, sxy, L));
-    return anti_bounce_back(r.kap, r.fac, gk, gi, gy_i, eq);
+    return anti_bounce_back(kap, fac, gk, gi, gy_i, eq);
 }
 
 // Populations f(x, t) of a boundary node: pulled where the link is intact,
