@@ -367,23 +367,37 @@ __device__ __forceinline__ void collide(float f[9], float sx, float sy, const La
 }
 
 // u(t+1) = u(t) + j/rho with Kahan compensation per component; w holds
-// (u_x, u_y, compensation_x, compensation_y).
+// (u_x, u_y, compensation_x, compensation_y).  kPaired: the two components in
+// pairs, bit by bit the scalar operations; k_interior takes them one by one,
+// which leaves it fewer spills in its 32 registers (one step in place of a
+// 1400^2 lattice 32.9 us with pairs, 32.5 without).
+template <bool kPaired = true>
 __device__ __forceinline__ void integrate_u_value(float4 &w, float jx, float jy, float rho) {
     // v = j/rho as j times one approximate reciprocal (relative error about
-    // 1e-7, far below the FP32 parity bound; no divisions); the two components
-    // in pairs (bit by bit the scalar operations)
+    // 1e-7, far below the FP32 parity bound; no divisions)
     float ir;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ir) : "f"(rho));
-    const F2 v = f2(rmul(jx, ir), rmul(jy, ir)), u = f2(w.x, w.y);
-    const F2 y = rsub(v, f2(w.z, w.w)), t = radd(u, y);
-    f2_split(rsub(rsub(t, u), y), w.z, w.w);
-    f2_split(t, w.x, w.y);
+    const float vx = rmul(jx, ir), vy = rmul(jy, ir);
+    if constexpr (kPaired) {
+        const F2 u = f2(w.x, w.y), y = rsub(f2(vx, vy), f2(w.z, w.w)), t = radd(u, y);
+        f2_split(rsub(rsub(t, u), y), w.z, w.w);
+        f2_split(t, w.x, w.y);
+    } else {
+        float y = rsub(vx, w.z), t = radd(w.x, y);
+        w.z = rsub(rsub(t, w.x), y);
+        w.x = t;
+        y = rsub(vy, w.w);
+        t = radd(w.y, y);
+        w.w = rsub(rsub(t, w.y), y);
+        w.y = t;
+    }
 }
 
 // 16-bit storage: u(t+1) = u(t) + j/rho without compensation; w holds
 // (u_x, u_y).  The populations' own rounding (FP16: 2^-11 of their size, each
 // step) is far larger than what the compensation recovers, and the record is
 // half as many bytes in the bandwidth-bound step.
+template <bool = true>
 __device__ __forceinline__ void integrate_u_value(float2 &w, float jx, float jy, float rho) {
     const float ir = __fdividef(1.0f, rho);
     w.x = radd(w.x, rmul(jx, ir));
@@ -1057,7 +1071,7 @@ __device__ __forceinline__ void interior_node(const T *src, T *dst, URec<T> *__r
         for (int i = 0; i < 9; ++i) m = fmaxf(m, fabsf(f[i]));
         note_range<T>(L, m);
     }
-    integrate_u_value(w, jx, jy, L.rho0 + dr);
+    integrate_u_value<kBatch>(w, jx, jy, L.rho0 + dr);
     uc[k] = w;
     flag_nonfinite(status, dr, jx, jy);
 }
