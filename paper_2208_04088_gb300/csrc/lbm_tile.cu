@@ -32,8 +32,8 @@
 // work in 2740).  On lattices of less than a few hundred thousand nodes it is
 // the latency of one step (two block barriers, the collision's and a link's
 // dependent chain: 2 us in a 32 x 32 tile) and of the launch.  2048^2 edge
-// crack, 500 steps: 11.7 ms (strips 18.9); with lambda != mu 21.5 (one step per
-// launch 44.8); 1024 x 512 plate with a hole, 600 steps: 2.52 (4.26).
+// crack, 500 steps: 11.7 ms (strips 18.9); with lambda != mu 21.7 (one step per
+// launch 44.8); 1024 x 512 plate with a hole, 600 steps: 2.57 (4.26).
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
