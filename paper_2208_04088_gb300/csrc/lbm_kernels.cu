@@ -63,13 +63,15 @@ __global__ void __launch_bounds__(kBT, 8) k_interior(const T *src, T *dst,
 }
 
 // 16-bit storage, two buffers, lambda = mu: two adjacent nodes per thread
-// (interior_pair).  Blocks of kBT threads the register bound aims at: FP16
-// measured fastest at six (40 registers: 93.9 against 90.4 GLUPS at four on the
-// 2048^2 crack), BF16 at four (100.7 against 98.9 at six).
-template <class T> constexpr int kPairMinBlocks = std::is_same<T, __half>::value ? 6 : 4;
+// (interior_pair), BX x BY threads to a block (pair_in_rows).  Threads per SM the
+// register bound aims at: FP16 measured fastest at 1536 (40 registers: 93.9
+// against 90.4 GLUPS at 1024 on the 2048^2 crack), BF16 at 1024 (100.7 against
+// 98.9 at 1536).  The shape is a constant of the kernel: with blockDim read
+// instead, 500 steps of the FP16 crack take 22.0 ms, 21.6 so.
+template <class T> constexpr int kPairThreads = std::is_same<T, __half>::value ? 1536 : 1024;
 
-template <class T>
-__global__ void __launch_bounds__(kBT, kPairMinBlocks<T>) k_interior_pair(const T *__restrict__ src,
+template <class T, int BX, int BY>
+__global__ void __launch_bounds__(BX *BY, kPairThreads<T> / (BX * BY)) k_interior_pair(const T *__restrict__ src,
                                                             T *__restrict__ dst,
                                                             float2 *__restrict__ uc,
                                                             const uint8_t *__restrict__ cls,
@@ -77,8 +79,8 @@ __global__ void __launch_bounds__(kBT, kPairMinBlocks<T>) k_interior_pair(const 
                                                             uint32_t *__restrict__ status,
                                                             const int64_t *__restrict__ time,
                                                             int toff) {
-    const int x0 = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int x0 = 2 * (int)(blockIdx.x * BX + threadIdx.x);
+    const int y = blockIdx.y * BY + (BY > 1 ? threadIdx.y : 0);
     // FP16: this step's scales.  The thread of node (0, 0), which is never
     // interior, publishes them after its node classes have been read, so that
     // no store sits between the loads of a thread and delays them.
@@ -410,13 +412,15 @@ static dim3 node_block(const Lattice &L) {
     const int64_t nodes = (int64_t)L.nx * L.ny;
     return L.nx >= 512 && nodes >= (L.in_place ? 1 << 18 : 1 << 20) ? dim3(128, 2) : dim3(32, 4);
 }
-// Blocks of two nodes per thread (16-bit storage): 64 x 1 beyond L2, where the
-// next block also finds its place as soon as two warps end.  32 x 4 / 64 x 1,
-// FP16: 520 x 1000 7.04 / 7.63, 800^2 7.68 / 8.03, 1024^2 10.05 / 10.12, 1400^2
-// 17.30 / 17.17, 2048^2 43.3 / 42.7 (32 x 8 44.4); BF16: 520 x 1000 5.98 / 6.42,
-// 1024^2 8.56 / 8.66, 1400^2 14.70 / 14.63, 2048^2 40.0 / 39.4.
-static dim3 pair_block(const Lattice &L) {
-    return L.nx >= 1024 && (int64_t)L.nx * L.ny > 1 << 20 ? dim3(64, 1) : dim3(32, 4);
+// Whether the blocks of two nodes per thread (16-bit storage) are 64 x 1 and
+// not 32 x 4: lattices that L2 does not hold (44 B per node), where the next
+// block also finds its place as soon as two warps end; below, the wider rows
+// idle more at the right edge.
+// 32 x 4 / 64 x 1, FP16: 520 x 1000 7.04 / 7.63, 800^2 7.68 / 8.03, 1024^2 10.05 /
+// 10.12, 1400^2 17.30 / 17.17, 2048^2 43.3 / 42.7 (32 x 8 44.4); BF16: 520 x 1000
+// 5.98 / 6.42, 1024^2 8.56 / 8.66, 1400^2 14.70 / 14.63, 2048^2 40.0 / 39.4.
+static bool pair_in_rows(const Lattice &L) {
+    return L.nx >= 1024 && (int64_t)L.nx * L.ny > 1 << 21;
 }
 
 template <class T>
@@ -431,9 +435,14 @@ static void launch_interior(const T *src, T *dst, const DevState &S, const Latti
     }
     if constexpr (!std::is_same<T, float>::value) {
         // 16-bit storage: two nodes per thread
-        const dim3 blk = pair_block(L);
-        k_interior_pair<T><<<lattice_grid(L, 2, blk), blk, 0, s>>>(
-            src, dst, static_cast<float2 *>(S.ucomp), S.cls, L, S.status, S.time, toff);
+        auto launch = [&](auto kernel, dim3 blk) {
+            kernel<<<lattice_grid(L, 2, blk), blk, 0, s>>>(
+                src, dst, static_cast<float2 *>(S.ucomp), S.cls, L, S.status, S.time, toff);
+        };
+        if (pair_in_rows(L))
+            launch(k_interior_pair<T, 64, 1>, dim3(64, 1));
+        else
+            launch(k_interior_pair<T, 32, 4>, dim3(32, 4));
         return;
     }
     // one row per thread measured fastest for every storage (2 and 4 rows cost

@@ -28,10 +28,10 @@ def _plate(nx, ny):
 
 
 @pytest.mark.parametrize("storage", ["f32", "f16"])
-@pytest.mark.parametrize("nx,ny", [(511, 513), (512, 512), (512, 511), (515, 517), (1024, 1024), (1027, 1025)])
+@pytest.mark.parametrize("nx,ny", [(511, 513), (512, 512), (512, 511), (515, 517), (1024, 1024), (1027, 1025), (1501, 1399)])
 def test_one_lattice(nx, ny, storage):
     """Both ends of the rules for in place (512 columns, 2^18 nodes) and for two
-    buffers (2^20 nodes, 16 bits beyond them and 1024 columns)."""
+    buffers (2^20 nodes, 16 bits beyond 2^21 and 1024 columns)."""
     from paper_2208_04088_gb300 import _native as N
     wl = _plate(nx, ny)
     two = _fields(N.desc_from_workload(wl, storage=storage, time_block=1), 37)
